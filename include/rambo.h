@@ -334,8 +334,10 @@ int rambo_copy_partition(const rambo_t *h, uint32_t *dst);
 typedef struct {
     uint32_t probe_ctas_per_sm;        /* probe grid = SMs x this; 0 = occupancy max */
     uint32_t probe_min_kmers_per_warp; /* smallest k-mer range a warp takes; 0 = 64  */
-    uint32_t expand_ctas_per_sm;       /* expansion grid cap = SMs x this (1..64)    */
-    uint32_t use_byte_table;           /* 1: expand through a per-8-bucket OR table  */
+    uint32_t expand_ctas_per_sm;       /* grid cap of the answer kernels (expansion   */
+                                       /* and single k-mers) = SMs x this (1..64)    */
+    uint32_t use_byte_table;           /* 1: path 1 expands a query through a         */
+                                       /* per-8-bucket OR table                       */
     uint32_t byte_table_max_mb;        /* ... only if it fits this many MiB          */
     uint32_t query_path;               /* sequence queries: 0 = prefix scan + probe +  */
                                        /* expand launches; 1 = persistent fused launch */
@@ -355,22 +357,19 @@ typedef struct {
     uint32_t fused_tile_kmers;         /* path 1: k-mers per tile of a long query      */
     uint32_t fused_short_max;          /* path 1: queries with at most this many       */
                                        /* k-mers are probed and expanded by one warp   */
-    uint32_t smem_docbits;             /* 1: expansion stages the bucket->document     */
-                                       /* bitmaps in shared memory when they fit       */
-    uint32_t use_nibble_table;         /* 1: expansion through a per-4-bucket OR table */
-                                       /* staged in shared memory, when it fits 96 KiB */
-    uint32_t expand_filter;            /* 1: expansion forms repetition 0's union and  */
-                                       /* then tests only surviving documents against  */
-                                       /* the later repetitions (needs the nibble      */
-                                       /* table, B <= 256 and a small K)               */
+    uint32_t smem_docbits;             /* no effect (0 or 1)                           */
+    uint32_t use_nibble_table;         /* no effect (0 or 1)                           */
+    uint32_t expand_filter;            /* no effect (0 or 1)                           */
     uint32_t early_exit;               /* path 1: stop probing a query once one of its */
                                        /* repetition rows is empty (its answer is then */
                                        /* empty; Section 3.3.1 "the first FALSE is     */
                                        /* conclusive", Section 5.1 RAMBO+).  Off by    */
                                        /* default: every k-mer is probed               */
     uint32_t early_exit_segment;       /* k-mers between checks (multiple of 128)      */
-    uint32_t kmer_probe_ctas_per_sm;   /* single-k-mer probe grid = SMs x this;        */
-                                       /* 0 = as probe_ctas_per_sm                     */
+    uint32_t kmer_probe_ctas_per_sm;   /* single-k-mer probe grid = SMs x this (R * B  */
+                                       /* of 16384 and more; other geometries probe    */
+                                       /* and answer in one launch, see                */
+                                       /* expand_ctas_per_sm); 0 = as probe_ctas_per_sm */
     uint32_t host_chunk_kmers;         /* host-buffer calls: k-mers per pipelined      */
                                        /* chunk (copy in, query, copy out); 0 = about  */
                                        /* 16 MiB of answers per chunk; the first chunk */
@@ -418,8 +417,7 @@ typedef struct {
                                        /* the probes' gathers land in shared memory    */
                                        /* (cp.async) instead of registers, so the      */
                                        /* launch needs fewer registers (default 0)     */
-    uint32_t kmer_async;               /* the same for the single k-mer probe (16-byte */
-                                       /* groups, eta <= 2; default 0)                 */
+    uint32_t kmer_async;               /* no effect (0 or 1)                           */
     uint32_t seg_cut_bits;             /* query_path 3: a k-mer whose order hash has   */
                                        /* this many low zero bits starts a segment     */
                                        /* (segments of about 2^bits k-mers, at least   */

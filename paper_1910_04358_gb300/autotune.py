@@ -28,19 +28,12 @@ CACHE_FILE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuning_ca
 KNOBS = (
     ("query_path", (0, 1, 2, 3)),
     ("branch_priority", (0, 1, 2)),
-    # expansion variant before its grid: a variant's best grid differs; the
-    # filter takes precedence over the nibble table, so it is decided first
-    ("expand_filter", (0, 1)),
-    ("use_nibble_table", (0, 1)),
     ("use_byte_table", (0, 1)),
-    ("smem_docbits", (0, 1)),
     ("expand_ctas_per_sm", (2, 4, 8, 16, 32)),
     # staged gathers before the fused grid: they pay off at a smaller grid
     # that leaves room for the k-mer branch beside it
     ("fused_async", (0, 1)),
     ("probe_ctas_per_sm", (0, 1, 2, 4, 8)),
-    ("kmer_async", (0, 1)),
-    ("kmer_probe_ctas_per_sm", (0, 1, 2, 3, 4)),
     ("bin_region_kib", (16384, 32768, 65536, 131072)),
     ("bin_rows", (1, 2, 4)),
     ("seg_cut_bits", (4, 5, 6, 7, 8)),

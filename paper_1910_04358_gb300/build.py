@@ -20,6 +20,7 @@ OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT_DIR, "librambo_gpu.so")
 
 SOURCES = ["rambo_api.cu", "rambo_kernels_probe.cu", "rambo_kernels_expand.cu",
+           "rambo_kernels_answers.cu",
            "rambo_kernels_fused.cu", "rambo_kernels_build.cu",
            "rambo_kernels_words.cu", "rambo_kernels_binned.cu",
            "rambo_kernels_insert_binned.cu", "rambo_kernels_segments.cu",

@@ -26,13 +26,13 @@ struct rambo {
     uint32_t *d_index;       // m * Gw words
     uint32_t *d_docbits;     // R * B * W words
     uint32_t *d_phi;         // K * R
+    uint32_t *d_slots;       // documents' slots for the answer kernels, or null (R * B too large)
     uint32_t *d_err;         // latched device error bits
     unsigned long long *d_probed;  // k-mers probed under early exit
     void *d_stage;           // host-call staging + workspace
     size_t stage_bytes;
     bool any_inserted;       // set by the first insert call
     uint32_t *d_tab;         // byte table for the expansion (or null)
-    uint32_t *d_ntab;        // nibble table for the expansion (or null)
     unsigned long long *d_bins;  // binned insert: records (insert_mode 3), or null
     uint32_t *d_bin_count;       // binned insert: per-bin counts and the unit counter
     uint64_t bins_records;       // records d_bins holds
@@ -186,19 +186,9 @@ int kmer_probe_grid(const rambo_t *h) {
 }
 
 // (Re)allocates or frees the byte table to match the tuning; the table is
-// rebuilt from the current bitmaps on the handle's stream.  The nibble table
-// (small enough for shared memory) is kept whenever it fits 96 KiB.
+// rebuilt from the current bitmaps on the handle's stream.
 int apply_bytetab(rambo_t *h) {
     const Geometry &g = h->g;
-    const uint64_t nbytes = nibtab_words(g.B, g.R, g.W) * 4;
-    if (nbytes <= 96 * 1024 && g.W <= 128) {
-        if (!h->d_ntab) RAMBO_TRY(cudaMalloc(&h->d_ntab, nbytes));
-        RAMBO_TRY(launch_build_nibtab(h->d_docbits, g.B, g.R, g.W, h->d_ntab, h->sm_count, h->stream));
-    } else if (h->d_ntab) {
-        RAMBO_TRY(cudaStreamSynchronize(h->stream));
-        cudaFree(h->d_ntab);
-        h->d_ntab = nullptr;
-    }
     const uint64_t bytes = bytetab_words(g.B, g.R, g.W) * 4;
     const bool want = h->tune.use_byte_table &&
                       bytes <= (uint64_t)h->tune.byte_table_max_mb * (1ull << 20);
@@ -360,6 +350,21 @@ Aligned align_packed(const uint8_t *packed, uint64_t packed_bytes) {
     return Aligned{packed - mis, packed_bytes + mis, (uint64_t)mis * 4};
 }
 
+ExpandArgs expand_args(const rambo_t *h, const uint32_t *acc, uint64_t n, uint32_t *out) {
+    const Geometry &g = h->g;
+    return ExpandArgs{acc, n, g.Gw, g.B, g.R, g.W, h->d_docbits, out, h->d_tab};
+}
+
+// Answers of n queries from their bucket masks: 32 queries at a time through
+// the document table where the geometry has one, else row by row.
+int expand_enqueue(rambo_t *h, uint64_t n, const uint32_t *acc, uint32_t *out, cudaStream_t s) {
+    StageScope sc(h, RAMBO_STAGE_EXPAND, s, 1);
+    const int blocks = h->sm_count * (int)h->tune.expand_ctas_per_sm;
+    if (h->d_slots) RAMBO_TRY(launch_answers(h->g, acc, n, h->d_slots, out, blocks, h->sm_count, s));
+    else RAMBO_TRY(launch_expand(expand_args(h, acc, n, out), blocks, s));
+    return RAMBO_OK;
+}
+
 // Items are [begins[i], ends[i]); a CSR batch passes (offsets, offsets + 1).
 // fused_ctas_cap > 0 caps the persistent fused launch at that many CTAs per
 // SM (so that other kernels of the same batch can run beside it).
@@ -420,12 +425,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
                 StageScope sc(h, RAMBO_STAGE_PROBE_SEQS, s, binned_launches());
                 RAMBO_TRY(launch_binned(ba, g, h->sm_count, s));
             }
-            ExpandArgs e{acc, n, g.Gw, g.B, g.R, g.W, h->d_docbits, out, h->d_tab, h->tune.smem_docbits,
-                         h->tune.use_nibble_table ? h->d_ntab : nullptr, h->d_phi, g.K,
-                         h->tune.expand_filter};
-            StageScope sc(h, RAMBO_STAGE_EXPAND, s, 1);
-            RAMBO_TRY(launch_expand(e, h->sm_count * (int)h->tune.expand_ctas_per_sm, h->sm_count, s));
-            return RAMBO_OK;
+            return expand_enqueue(h, n, acc, out, s);
         }
     }
     if (use_segments(h) && ends == offsets + 1) {
@@ -484,12 +484,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
                                              reinterpret_cast<uint64_t *>(sw + S.sbsum_off), h->d_err, s));
                 RAMBO_TRY(launch_seg_probe(sa, g, h->sm_count, s));
             }
-            ExpandArgs e{acc, n, g.Gw, g.B, g.R, g.W, h->d_docbits, out, h->d_tab, h->tune.smem_docbits,
-                         h->tune.use_nibble_table ? h->d_ntab : nullptr, h->d_phi, g.K,
-                         h->tune.expand_filter};
-            StageScope sc(h, RAMBO_STAGE_EXPAND, s, 1);
-            RAMBO_TRY(launch_expand(e, h->sm_count * (int)h->tune.expand_ctas_per_sm, h->sm_count, s));
-            return RAMBO_OK;
+            return expand_enqueue(h, n, acc, out, s);
         }
     }
     if (h->tune.query_path >= 1 && fused_supported(g)) {
@@ -509,9 +504,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
         a.ends = ends;
         a.n = n;
         a.err = h->d_err;
-        ExpandArgs e{acc, n, g.Gw, g.B, g.R, g.W, h->d_docbits, out, h->d_tab, h->tune.smem_docbits,
-                     h->tune.use_nibble_table ? h->d_ntab : nullptr, h->d_phi, g.K,
-                     h->tune.expand_filter};
+        const ExpandArgs e = expand_args(h, acc, n, out);
         FusedQueues qs{};
         qs.counters = reinterpret_cast<uint32_t *>(w + L.qcnt);
         qs.short_list = reinterpret_cast<uint32_t *>(w + L.slist);
@@ -564,21 +557,14 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
         StageScope sc(h, RAMBO_STAGE_PROBE_SEQS, s, 1);
         RAMBO_TRY(launch_probe_seqs(a, g, probe_grid(h), s));
     }
-    ExpandArgs e{acc, n, g.Gw, g.B, g.R, g.W, h->d_docbits, out, h->d_tab, h->tune.smem_docbits,
-                     h->tune.use_nibble_table ? h->d_ntab : nullptr, h->d_phi, g.K,
-                     h->tune.expand_filter};
-    {
-        StageScope sc(h, RAMBO_STAGE_EXPAND, s, 1);
-        RAMBO_TRY(launch_expand(e, h->sm_count * (int)h->tune.expand_ctas_per_sm, h->sm_count, s));
-    }
-    return RAMBO_OK;
+    return expand_enqueue(h, n, acc, out, s);
 }
 
 int query_kmers_enqueue(rambo_t *h, uint64_t n, const uint64_t *kmers, uint32_t *out, void *ws,
                         cudaStream_t s) {
     const Geometry &g = h->g;
     uint32_t *acc = static_cast<uint32_t *>(ws);
-    if (g.eta > 4) RAMBO_TRY(cudaMemsetAsync(acc, 0xFF, n * (uint64_t)g.Gw * 4, s));
+    if (!h->d_slots && g.eta > 4) RAMBO_TRY(cudaMemsetAsync(acc, 0xFF, n * (uint64_t)g.Gw * 4, s));
     ProbeArgs a{};
     a.index = h->d_index;
     a.m = g.m;
@@ -592,18 +578,17 @@ int query_kmers_enqueue(rambo_t *h, uint64_t n, const uint64_t *kmers, uint32_t 
     a.acc = acc;
     a.err = h->d_err;
     a.min_chunk = h->tune.probe_min_kmers_per_warp;
+    if (h->d_slots) {  // probe and answer in one launch
+        StageScope sc(h, RAMBO_STAGE_PROBE_KMERS, s, 1);
+        RAMBO_TRY(launch_kmer_answers(a, g, h->d_slots, out, h->sm_count * (int)h->tune.expand_ctas_per_sm,
+                                      h->sm_count, s));
+        return RAMBO_OK;
+    }
     {
         StageScope sc(h, RAMBO_STAGE_PROBE_KMERS, s, 1);
-        RAMBO_TRY(launch_probe_kmers(a, g, kmer_probe_grid(h), s, h->tune.kmer_async != 0));
+        RAMBO_TRY(launch_probe_kmers(a, g, kmer_probe_grid(h), s));
     }
-    ExpandArgs e{acc, n, g.Gw, g.B, g.R, g.W, h->d_docbits, out, h->d_tab, h->tune.smem_docbits,
-                     h->tune.use_nibble_table ? h->d_ntab : nullptr, h->d_phi, g.K,
-                     h->tune.expand_filter};
-    {
-        StageScope sc(h, RAMBO_STAGE_EXPAND, s, 1);
-        RAMBO_TRY(launch_expand(e, h->sm_count * (int)h->tune.expand_ctas_per_sm, h->sm_count, s));
-    }
-    return RAMBO_OK;
+    return expand_enqueue(h, n, acc, out, s);
 }
 
 // Documents are [begins[i], ends[i]); a CSR batch passes (offsets, offsets +
@@ -622,7 +607,8 @@ int insert_enqueue(rambo_t *h, uint64_t n, const uint32_t *doc_ids, const uint8_
     const Aligned al = align_packed(packed, packed_bytes);
     {
         StageScope sc(h, RAMBO_STAGE_REGISTER, s, 1);
-        RAMBO_TRY(launch_register_docs(doc_ids, n, h->d_phi, g.K, g.R, g.B, g.W, h->d_docbits, h->d_err, s));
+        RAMBO_TRY(launch_register_docs(doc_ids, n, h->d_phi, g.K, g.R, g.B, g.W, h->d_docbits, h->d_slots,
+                                       h->d_err, s));
     }
     {
         StageScope sc(h, RAMBO_STAGE_PREFIX, s, kmer_prefix_launches(n));
@@ -678,10 +664,6 @@ int insert_enqueue(rambo_t *h, uint64_t n, const uint32_t *doc_ids, const uint8_
     if (h->d_tab) {
         StageScope sc(h, RAMBO_STAGE_REGISTER, s, 1);
         RAMBO_TRY(launch_build_bytetab(h->d_docbits, g.B, g.R, g.W, h->d_tab, h->sm_count, s));
-    }
-    if (h->d_ntab) {
-        StageScope sc(h, RAMBO_STAGE_REGISTER, s, 1);
-        RAMBO_TRY(launch_build_nibtab(h->d_docbits, g.B, g.R, g.W, h->d_ntab, h->sm_count, s));
     }
     return RAMBO_OK;
 }
@@ -949,6 +931,10 @@ int rambo_create(uint32_t K, uint32_t B, uint32_t R, uint64_t m, uint32_t eta, u
     if ((rc = cuda_rc(cudaMalloc(&h->d_index, index_bytes)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&h->d_docbits, docbits_bytes)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&h->d_phi, (uint64_t)K * R * 4)))) return fail(rc);
+    if (const uint64_t words = answer_slot_words(h->g)) {
+        if ((rc = cuda_rc(cudaMalloc(&h->d_slots, words * 4)))) return fail(rc);
+        if ((rc = cuda_rc(launch_slots(h->g, h->d_slots, nullptr, nullptr, h->sm_count, h->stream)))) return fail(rc);
+    }
     if ((rc = cuda_rc(cudaMalloc(&h->d_err, 4)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&h->d_probed, 8)))) return fail(rc);
     if ((rc = cuda_rc(cudaMemsetAsync(h->d_probed, 0, 8, h->stream)))) return fail(rc);
@@ -999,11 +985,11 @@ int rambo_destroy(rambo_t *h) {
     cudaFree(h->d_index);
     cudaFree(h->d_docbits);
     cudaFree(h->d_phi);
+    cudaFree(h->d_slots);
     cudaFree(h->d_err);
     cudaFree(h->d_probed);
     cudaFree(h->d_stage);
     cudaFree(h->d_tab);
-    cudaFree(h->d_ntab);
     cudaFree(h->d_bins);
     cudaFree(h->d_bin_count);
     for (auto &p : h->pending) {
@@ -1271,7 +1257,7 @@ int rambo_insert_words_dev(rambo_t *h, uint32_t n_docs, const uint32_t *doc_ids,
     {
         StageScope sc(h, RAMBO_STAGE_REGISTER, s, 1);
         RAMBO_TRY(launch_register_docs(doc_ids, n_docs, h->d_phi, g.K, g.R, g.B, g.W, h->d_docbits,
-                                       h->d_err, s));
+                                       h->d_slots, h->d_err, s));
     }
     WordArgs a{};
     a.index = h->d_index;
@@ -1292,7 +1278,6 @@ int rambo_insert_words_dev(rambo_t *h, uint32_t n_docs, const uint32_t *doc_ids,
         RAMBO_TRY(launch_insert_words(a, h->sm_count, s));
     }
     if (h->d_tab) RAMBO_TRY(launch_build_bytetab(h->d_docbits, g.B, g.R, g.W, h->d_tab, h->sm_count, s));
-    if (h->d_ntab) RAMBO_TRY(launch_build_nibtab(h->d_docbits, g.B, g.R, g.W, h->d_ntab, h->sm_count, s));
     return RAMBO_OK;
 }
 
@@ -1332,13 +1317,7 @@ int rambo_query_words_dev(rambo_t *h, uint64_t n, const uint8_t *bytes, uint64_t
         StageScope sc(h, RAMBO_STAGE_PROBE_SEQS, s, 1);
         RAMBO_TRY(launch_probe_words(a, h->sm_count, s));
     }
-    ExpandArgs e{acc, n, g.Gw, g.B, g.R, g.W, h->d_docbits, out, h->d_tab, h->tune.smem_docbits,
-                 h->tune.use_nibble_table ? h->d_ntab : nullptr, h->d_phi, g.K, h->tune.expand_filter};
-    {
-        StageScope sc(h, RAMBO_STAGE_EXPAND, s, 1);
-        RAMBO_TRY(launch_expand(e, h->sm_count * (int)h->tune.expand_ctas_per_sm, h->sm_count, s));
-    }
-    return RAMBO_OK;
+    return expand_enqueue(h, n, acc, out, s);
 }
 
 // -------------------------------------------------------- explicit partition
@@ -1366,7 +1345,7 @@ int rambo_fold(rambo_t *h) {
     DeviceGuard guard(h->device);
     if (!guard.ok) return RAMBO_ECUDA;
     RAMBO_TRY(cudaStreamSynchronize(h->stream));
-    uint32_t *ni = nullptr, *nd = nullptr, *np = nullptr;
+    uint32_t *ni = nullptr, *nd = nullptr, *np = nullptr, *ns = nullptr;
     const uint64_t ni_bytes = ng.m * (uint64_t)ng.Gw * 4;
     const uint64_t nd_bytes = (uint64_t)ng.R * ng.B * ng.W * 4;
     int rc = cuda_rc(cudaMalloc(&ni, ni_bytes));
@@ -1376,16 +1355,23 @@ int rambo_fold(rambo_t *h) {
                                       nd, old.W, h->sm_count, h->stream));
     // the folded partition is phi_r(d) mod B/2 = hash mod B/2, since B/2 divides B
     if (!rc) rc = cuda_rc(launch_partition(np, ng.K, ng.R, ng.B, ng.seed, h->stream));
+    // the documents' slots of the folded geometry
+    const uint64_t slot_words = answer_slot_words(ng);
+    if (!rc && slot_words) rc = cuda_rc(cudaMalloc(&ns, slot_words * 4));
+    if (!rc && slot_words) rc = cuda_rc(launch_slots(ng, ns, nd, np, h->sm_count, h->stream));
     if (!rc) rc = cuda_rc(cudaStreamSynchronize(h->stream));
     if (rc) {
         cudaFree(ni);
         cudaFree(nd);
         cudaFree(np);
+        cudaFree(ns);
         return rc;  // the index is unchanged
     }
     cudaFree(h->d_index);
     cudaFree(h->d_docbits);
     cudaFree(h->d_phi);
+    cudaFree(h->d_slots);
+    h->d_slots = ns;
     h->d_index = ni;
     h->d_docbits = nd;
     h->d_phi = np;
@@ -1393,10 +1379,6 @@ int rambo_fold(rambo_t *h) {
     if (h->d_tab) {
         cudaFree(h->d_tab);
         h->d_tab = nullptr;
-    }
-    if (h->d_ntab) {
-        cudaFree(h->d_ntab);
-        h->d_ntab = nullptr;
     }
     return apply_bytetab(h);
 }

@@ -195,11 +195,6 @@ struct ExpandArgs {
     const uint32_t *docbits; // R*B*W
     uint32_t *out;           // n x W
     const uint32_t *tab;     // byte table (R*ceil(B/8)*256*W) or null
-    uint32_t smem_docbits;   // 1: stage DocBits in shared memory when it fits
-    const uint32_t *ntab;    // nibble table (R*ceil(B/4)*16*W) or null
-    const uint32_t *phi;     // K x R partition (candidate filtering)
-    uint32_t K;
-    uint32_t filter;         // 1: expand by candidate filtering when it fits
 };
 
 struct InsertArgs {
@@ -263,9 +258,10 @@ cudaError_t launch_kmer_prefix(const uint64_t *begins, const uint64_t *ends, uin
                                uint32_t *err, cudaStream_t s, uint32_t tile = 0,
                                uint32_t short_max = 0);
 size_t kmer_prefix_block_sums(uint64_t n);
+// (slots: the answer kernels' document table, or null)
 cudaError_t launch_register_docs(const uint32_t *doc_ids, uint64_t n, const uint32_t *phi,
                                  uint32_t K, uint32_t R, uint32_t B, uint32_t W, uint32_t *docbits,
-                                 uint32_t *err, cudaStream_t s);
+                                 uint32_t *slots, uint32_t *err, cudaStream_t s);
 cudaError_t launch_insert(const InsertArgs &a, int sm_count, cudaStream_t s);
 // ORs the answers of one document shard (n rows of shard_words words, bit j
 // = the shard's local document j) into global answer rows of out_words
@@ -279,9 +275,8 @@ cudaError_t launch_fold(const uint32_t *old_index, uint32_t old_gw, uint32_t *ne
                         const uint32_t *old_db, uint32_t *new_db, uint32_t W, int sm_count,
                         cudaStream_t s);
 cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, int sm_count, cudaStream_t s);
-// staged: one-lane 16-byte groups and eta <= 2 gather into shared memory (cp.async)
-cudaError_t launch_probe_kmers(const ProbeArgs &a, const Geometry &g, int sm_count, cudaStream_t s,
-                               bool staged);
+// (groups of 512 bytes and more; the others are probed by launch_kmer_answers)
+cudaError_t launch_probe_kmers(const ProbeArgs &a, const Geometry &g, int sm_count, cudaStream_t s);
 // Work queues of the persistent fused query (workspace arrays).
 struct FusedQueues {
     uint32_t *counters;      // 8 words, zeroed by the launcher
@@ -370,14 +365,30 @@ cudaError_t launch_seg_probe(const SegArgs &a, const Geometry &g, int sm_count, 
 cudaError_t launch_fused(const ProbeArgs &p, const ExpandArgs &e, const Geometry &g,
                          const FusedQueues &qs, int grid_override, int sm_count, cudaStream_t s);
 
+// Answers for 32 queries at a time (rambo_kernels_answers.cu).  The document
+// table holds for every document d and repetition r the slot r*B + phi_r(d)
+// of its bucket as a 16-bit byte offset (4 x slot), or the empty slot R*B for
+// documents that are not inserted; documents are padded to a multiple of 128.
+__host__ __device__ inline uint64_t answer_slot_index(uint32_t d, uint32_t r, uint32_t R) {
+    return (((uint64_t)(d >> 5) * ((R + 1) / 2) + r / 2) * 32 + (d & 31)) * 2 + (r & 1);
+}
+// 32-bit words of the table; 0 when R*B is too large for it.
+uint64_t answer_slot_words(const Geometry &g);
+// Empties the table; with docbits, then enters every inserted document.
+cudaError_t launch_slots(const Geometry &g, uint32_t *slots, const uint32_t *docbits, const uint32_t *phi,
+                         int sm_count, cudaStream_t s);
+// Answers of n queries from their bucket masks acc (n x Gw).
+cudaError_t launch_answers(const Geometry &g, const uint32_t *acc, uint64_t n, const uint32_t *slots, uint32_t *out,
+                           int max_blocks, int sm_count, cudaStream_t s);
+// Single k-mers probed and answered in one launch (p: index, hashing, k-mers).
+cudaError_t launch_kmer_answers(const ProbeArgs &p, const Geometry &g, const uint32_t *slots, uint32_t *out,
+                                int max_blocks, int sm_count, cudaStream_t s);
+
 // max_blocks caps the expansion grid
-cudaError_t launch_expand(const ExpandArgs &a, int max_blocks, int sm_count, cudaStream_t s);
+cudaError_t launch_expand(const ExpandArgs &a, int max_blocks, cudaStream_t s);
 // A bounded mbarrier wait that nothing completes; latches ERR_WAIT on expiry.
 cudaError_t launch_wait_expiry(uint32_t *err, uint64_t spins, cudaStream_t s);
 uint64_t bytetab_words(uint32_t B, uint32_t R, uint32_t W);
-uint64_t nibtab_words(uint32_t B, uint32_t R, uint32_t W);
-cudaError_t launch_build_nibtab(const uint32_t *docbits, uint32_t B, uint32_t R, uint32_t W,
-                                uint32_t *ntab, int sm_count, cudaStream_t s);
 cudaError_t launch_build_bytetab(const uint32_t *docbits, uint32_t B, uint32_t R, uint32_t W,
                                  uint32_t *tab, int sm_count, cudaStream_t s);
 

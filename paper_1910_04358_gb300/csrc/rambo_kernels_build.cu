@@ -172,7 +172,8 @@ k_prefix_single(const uint64_t *begins, const uint64_t *ends, uint64_t n, uint32
 
 // ------------------------------------------------------------- registration
 __global__ void k_register(const uint32_t *doc_ids, uint64_t n, const uint32_t *phi, uint32_t K,
-                           uint32_t R, uint32_t B, uint32_t W, uint32_t *docbits, uint32_t *err) {
+                           uint32_t R, uint32_t B, uint32_t W, uint32_t *docbits, uint16_t *slots,
+                           uint32_t *err) {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n * R) return;
     const uint64_t item = i / R;
@@ -184,6 +185,7 @@ __global__ void k_register(const uint32_t *doc_ids, uint64_t n, const uint32_t *
     }
     const uint32_t b = phi[(uint64_t)d * R + r];
     atomicOr(&docbits[((uint64_t)r * B + b) * W + (d >> 5)], 1u << (d & 31));
+    if (slots) slots[answer_slot_index(d, r, R)] = (uint16_t)(4 * (r * B + b));
 }
 
 // ------------------------------------------------------------------- insert
@@ -397,11 +399,11 @@ cudaError_t launch_kmer_prefix(const uint64_t *begins, const uint64_t *ends, uin
 
 cudaError_t launch_register_docs(const uint32_t *doc_ids, uint64_t n, const uint32_t *phi,
                                  uint32_t K, uint32_t R, uint32_t B, uint32_t W, uint32_t *docbits,
-                                 uint32_t *err, cudaStream_t s) {
+                                 uint32_t *slots, uint32_t *err, cudaStream_t s) {
     const uint64_t total = n * R;
     if (total == 0) return cudaSuccess;
     k_register<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(doc_ids, n, phi, K, R, B, W, docbits,
-                                                               err);
+                                                               reinterpret_cast<uint16_t *>(slots), err);
     return cudaGetLastError();
 }
 

@@ -88,7 +88,6 @@ __device__ __forceinline__ void warp_range(uint64_t T, uint32_t min_chunk, uint6
 // The answer is the AND of the R unions; a repetition with no passing bucket,
 // or an all-zero running AND, ends the unit early.
 constexpr int EXPAND_THREADS = 256;
-constexpr size_t SMEM_DOCBITS_MAX = 96 * 1024;
 
 // Byte j of repetition r's bucket row (buckets 8j .. 8j+7), masked to B.
 // (bm may point to global or shared memory.)
@@ -199,57 +198,6 @@ __device__ __forceinline__ void expand_unit_sparse(const ExpandArgs &a, const ui
             for (int t = 0; t < 8; ++t)
 #pragma unroll
                 for (int c = 0; c < C; ++c) o[c] |= val[t][c];
-        }
-        uint32_t nz = 0;
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            res[c] &= o[c];
-            nz |= res[c];
-        }
-        if (!any || !__any_sync(FULL, nz)) dead = true;
-    }
-    uint32_t *out = a.out + q * a.W;
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-        const uint32_t w = w0 + 32 * c;
-        if (w < a.W) out[w] = dead ? 0u : res[c];
-    }
-}
-
-// Union per repetition from DocBits staged in shared memory (sdb): each set
-// bit of the bucket row, taken 32 buckets at a time, ORs one row of W words
-// (consecutive words per lane: no bank conflicts).
-template <int C>
-__device__ __forceinline__ void expand_unit_smem(const ExpandArgs &a, const uint32_t *sdb,
-                                                 const uint32_t *bm, uint64_t q, uint32_t w0) {
-    uint32_t res[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) res[c] = FULL;
-    bool dead = false;
-    for (uint32_t r = 0; r < a.R && !dead; ++r) {
-        uint32_t o[C];
-#pragma unroll
-        for (int c = 0; c < C; ++c) o[c] = 0;
-        bool any = false;
-        const uint32_t lo = r * a.B;
-        for (uint32_t i = 0; i < a.B; i += 32) {
-            const uint32_t bit = lo + i;
-            const uint32_t wi = bit >> 5, sh = bit & 31;
-            uint32_t x = bm[wi];
-            if (sh) x = __funnelshift_r(x, wi + 1 < a.Gw ? bm[wi + 1] : 0u, sh);
-            const uint32_t nb = a.B - i < 32 ? a.B - i : 32;
-            if (nb < 32) x &= (1u << nb) - 1u;
-            any |= x != 0;
-            while (x) {
-                const uint32_t b = i + __ffs(x) - 1;
-                x &= x - 1;
-                const uint32_t *row = sdb + (lo + b) * a.W;
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const uint32_t w = w0 + 32 * c;
-                    if (w < a.W) o[c] |= row[w];
-                }
-            }
         }
         uint32_t nz = 0;
 #pragma unroll
