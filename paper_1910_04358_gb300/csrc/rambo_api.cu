@@ -26,6 +26,7 @@ struct rambo {
     uint32_t *d_index;       // m * Gw words
     uint32_t *d_docbits;     // R * B * W words
     uint32_t *d_phi;         // K * R
+    unsigned long long *d_pattern;  // documents' group words for insertion, or null
     uint32_t *d_slots;       // documents' slots for the answer kernels, or null (R * B too large)
     uint32_t *d_err;         // latched device error bits
     unsigned long long *d_probed;  // k-mers probed under early exit
@@ -634,10 +635,12 @@ int insert_enqueue(rambo_t *h, uint64_t n, const uint32_t *doc_ids, const uint8_
     a.kcum = kcum;
     a.n = n;
     a.err = h->d_err;
-    a.mode = h->tune.insert_mode;
+    a.pattern = h->d_pattern;
+    a.kind = !h->d_pattern ? 0 : g.Gw > 1 ? 1 : 2;
+    a.lanes = a.kind == 0 ? (g.R < 32 ? g.R : 32) : g.Gw > 1 ? g.Gw / 2 : 1;
     uint32_t rshift = 0;
     uint32_t nbins =
-        a.mode == 3 && h->d_bins && ends == offsets + 1
+        h->tune.insert_mode == 3 && h->d_bins && ends == offsets + 1
             ? binned_insert_bins(g.m, g.Gw * 4, g.K,
                                  (uint64_t)(h->tune.bin_region_kib ? h->tune.bin_region_kib : 32768) * 1024,
                                  &rshift)
@@ -657,7 +660,6 @@ int insert_enqueue(rambo_t *h, uint64_t n, const uint32_t *doc_ids, const uint8_
             RAMBO_TRY(launch_insert_binned(a, b, f0, f0 + per, h->sm_count, s));
         }
     } else {
-        if (a.mode == 3) a.mode = 2;  // too many regions, or too many chunks
         StageScope sc(h, RAMBO_STAGE_INSERT, s, 1);
         RAMBO_TRY(launch_insert(a, h->sm_count, s));
     }
@@ -942,6 +944,10 @@ int rambo_create(uint32_t K, uint32_t B, uint32_t R, uint64_t m, uint32_t eta, u
     if ((rc = cuda_rc(cudaMemsetAsync(h->d_docbits, 0, docbits_bytes, h->stream)))) return fail(rc);
     if ((rc = cuda_rc(cudaMemsetAsync(h->d_err, 0, 4, h->stream)))) return fail(rc);
     if ((rc = cuda_rc(launch_partition(h->d_phi, K, R, B, seed, h->stream)))) return fail(rc);
+    if (const uint64_t bytes = pattern_bytes(h->g)) {
+        if ((rc = cuda_rc(cudaMalloc(&h->d_pattern, bytes)))) return fail(rc);
+        if ((rc = cuda_rc(launch_patterns(h->g, h->d_pattern, h->d_phi, h->stream)))) return fail(rc);
+    }
     if ((rc = cuda_rc(cudaStreamSynchronize(h->stream)))) return fail(rc);
     h->tune.probe_ctas_per_sm = 0;
     h->tune.probe_min_kmers_per_warp = 0;
@@ -986,6 +992,7 @@ int rambo_destroy(rambo_t *h) {
     cudaFree(h->d_docbits);
     cudaFree(h->d_phi);
     cudaFree(h->d_slots);
+    cudaFree(h->d_pattern);
     cudaFree(h->d_err);
     cudaFree(h->d_probed);
     cudaFree(h->d_stage);
@@ -1332,6 +1339,10 @@ int rambo_set_partition(rambo_t *h, const uint32_t *phi) {
     if (!guard.ok) return RAMBO_ECUDA;
     RAMBO_TRY(cudaStreamSynchronize(h->stream));
     RAMBO_TRY(cudaMemcpy(h->d_phi, phi, n * 4, cudaMemcpyHostToDevice));
+    if (h->d_pattern) {
+        RAMBO_TRY(launch_patterns(h->g, h->d_pattern, h->d_phi, h->stream));
+        RAMBO_TRY(cudaStreamSynchronize(h->stream));
+    }
     return RAMBO_OK;
 }
 
@@ -1346,6 +1357,7 @@ int rambo_fold(rambo_t *h) {
     if (!guard.ok) return RAMBO_ECUDA;
     RAMBO_TRY(cudaStreamSynchronize(h->stream));
     uint32_t *ni = nullptr, *nd = nullptr, *np = nullptr, *ns = nullptr;
+    unsigned long long *pt = nullptr;
     const uint64_t ni_bytes = ng.m * (uint64_t)ng.Gw * 4;
     const uint64_t nd_bytes = (uint64_t)ng.R * ng.B * ng.W * 4;
     int rc = cuda_rc(cudaMalloc(&ni, ni_bytes));
@@ -1359,12 +1371,16 @@ int rambo_fold(rambo_t *h) {
     const uint64_t slot_words = answer_slot_words(ng);
     if (!rc && slot_words) rc = cuda_rc(cudaMalloc(&ns, slot_words * 4));
     if (!rc && slot_words) rc = cuda_rc(launch_slots(ng, ns, nd, np, h->sm_count, h->stream));
+    const uint64_t pt_bytes = pattern_bytes(ng);
+    if (!rc && pt_bytes) rc = cuda_rc(cudaMalloc(&pt, pt_bytes));
+    if (!rc && pt_bytes) rc = cuda_rc(launch_patterns(ng, pt, np, h->stream));
     if (!rc) rc = cuda_rc(cudaStreamSynchronize(h->stream));
     if (rc) {
         cudaFree(ni);
         cudaFree(nd);
         cudaFree(np);
         cudaFree(ns);
+        cudaFree(pt);
         return rc;  // the index is unchanged
     }
     cudaFree(h->d_index);
@@ -1372,6 +1388,8 @@ int rambo_fold(rambo_t *h) {
     cudaFree(h->d_phi);
     cudaFree(h->d_slots);
     h->d_slots = ns;
+    cudaFree(h->d_pattern);
+    h->d_pattern = pt;
     h->d_index = ni;
     h->d_docbits = nd;
     h->d_phi = np;

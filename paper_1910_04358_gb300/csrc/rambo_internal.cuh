@@ -211,8 +211,10 @@ struct InsertArgs {
     const uint64_t *kcum;      // n+1
     uint64_t n;
     uint32_t *err;
-    uint32_t mode;             // 0: warp-aggregated 32-bit atomics; 1: plain 32-bit;
-                               // 2: plain, repetitions sharing a 64-bit word merged
+    const unsigned long long *pattern;  // pattern_bytes: the documents' group words, or null
+    uint32_t kind;             // RecordSetter: 0 = a lane per repetition, 1 = per 64-bit word,
+                               // 2 = one 32-bit word
+    uint32_t lanes;            // lanes per record
 };
 
 // Word documents (Section 5.4): term t is bytes [term_offs[t], term_offs[t+1])
@@ -263,6 +265,14 @@ cudaError_t launch_register_docs(const uint32_t *doc_ids, uint64_t n, const uint
                                  uint32_t K, uint32_t R, uint32_t B, uint32_t W, uint32_t *docbits,
                                  uint32_t *slots, uint32_t *err, cudaStream_t s);
 cudaError_t launch_insert(const InsertArgs &a, int sm_count, cudaStream_t s);
+// Bytes of the documents' patterns (every word of a document's group bits)
+// where records are set word by word: 4-byte groups, and groups of at most R
+// 32-bit words, where a lane per 64-bit word needs at most half the lanes of
+// one per repetition (16-byte groups with R = 4 in L2: 207 against 201 G
+// records/s).  Wider groups give 0 and are set repetition by repetition
+// (32-byte groups with R = 5: 151 against 130; equal in DRAM).
+uint64_t pattern_bytes(const Geometry &g);
+cudaError_t launch_patterns(const Geometry &g, unsigned long long *pattern, const uint32_t *phi, cudaStream_t s);
 // ORs the answers of one document shard (n rows of shard_words words, bit j
 // = the shard's local document j) into global answer rows of out_words
 // words at bit global_ids[j] (device array of shard_docs ids).

@@ -9,9 +9,8 @@
 //   insert     Algorithm 1: every k-mer x of document d sets bits
 //              h_1(x)..h_eta(x) of BFU (phi_r(d), r) for every r.  In the
 //              bit-sliced layout that is bit r*B+phi_r(d) of position group
-//              h_j(x); lanes of a warp that hit the same word are combined
-//              (warp-aggregated atomicOr) before one atomic is issued.
-#include "rambo_internal.cuh"
+//              h_j(x), set with one atomicOr per repetition or 64-bit word.
+#include "rambo_insert_common.cuh"
 
 namespace rgpu {
 namespace {
@@ -191,12 +190,11 @@ __global__ void k_register(const uint32_t *doc_ids, uint64_t n, const uint32_t *
 // ------------------------------------------------------------------- insert
 constexpr int INSERT_THREADS = 256;
 
-// MODE 0: lanes that hit the same index word combine their bits first
-// (match + OR-reduce) and one of them issues the atomic; MODE 1: every
-// (k-mer, probe, repetition) issues its own atomicOr; MODE 2: as 1, but the
-// bits of consecutive repetitions that fall into one 64-bit word go in one
-// 64-bit atomicOr (the repetitions' bits r*B + phi_r(d) ascend with r).
-template <int ETA, int MODE>
+// Each warp walks a contiguous range of the flat k-mer index, 32 k-mers at a
+// time; every lane hashes one k-mer, then the warp sets the 32 records of
+// each probe together (RecordSetter).  Bound by DRAM once the index outgrows
+// L2: every record reads and writes back the lines of its group.
+template <int ETA, int KIND>
 __global__ void __launch_bounds__(INSERT_THREADS, 1) k_insert(InsertArgs a) {
     const int lane = threadIdx.x & 31;
     const uint64_t T = a.kcum[a.n];
@@ -217,19 +215,19 @@ __global__ void __launch_bounds__(INSERT_THREADS, 1) k_insert(InsertArgs a) {
         else hi = mid;
     }
     const uint64_t i_first = lo;
+    RecordSetter<KIND> set(a, lane);
 
     for (uint32_t jb = 0; jb < a.eta; jb += ETA) {
         uint64_t item = i_first;
         for (uint64_t base = c0; base < c1; base += 32) {
             const uint64_t g = base + lane;
-            bool val = g < c1;
-            uint32_t d = 0;
+            uint32_t d = NO_DOC;
             uint64_t c = 0;
-            if (val) {
+            if (g < c1) {
                 while (a.kcum[item + 1] <= g) ++item;
                 d = a.doc_ids[item];
                 if (d >= a.K) {
-                    val = false;
+                    d = NO_DOC;
                 } else {
                     const uint64_t start = a.offsets[item] + a.base_shift + (g - a.kcum[item]);
                     c = canonical_from_window(base_window(a.packed, a.packed_bytes, start), a.k);
@@ -240,45 +238,28 @@ __global__ void __launch_bounds__(INSERT_THREADS, 1) k_insert(InsertArgs a) {
             for (int e = 0; e < ETA; ++e) {
                 if (jb + e >= a.eta) break;  // warp-uniform
                 const uint64_t h = mh_first_word(km, a.seed32 + jb + e);
-                const uint64_t p = a.m_pow2 ? (h & (a.m - 1)) : (h % a.m);
-                if (MODE == 0) {
-                    for (uint32_t r = 0; r < a.R; ++r) {
-                        uint64_t addr = ~0ULL;
-                        uint32_t bit = 0;
-                        if (val) {
-                            const uint32_t bb = r * a.B + a.phi[(uint64_t)d * a.R + r];
-                            addr = p * a.Gw + (bb >> 5);
-                            bit = 1u << (bb & 31);
-                        }
-                        const uint32_t peers = __match_any_sync(FULL, addr);
-                        const uint32_t v = __reduce_or_sync(peers, bit);
-                        if (val && lane == __ffs(peers) - 1) atomicOr(a.index + addr, v);
-                    }
-                } else if (val) {
-                    const uint64_t gbit = p * a.Gw * 32;  // first bit of the group
-                    if (MODE == 1) {
-                        for (uint32_t r = 0; r < a.R; ++r) {
-                            const uint64_t bb = gbit + r * a.B + a.phi[(uint64_t)d * a.R + r];
-                            atomicOr(a.index + (bb >> 5), 1u << (bb & 31));
-                        }
-                    } else {
-                        unsigned long long *idx64 = reinterpret_cast<unsigned long long *>(a.index);
-                        uint64_t cur = ~0ULL, bits = 0;
-                        for (uint32_t r = 0; r < a.R; ++r) {
-                            const uint64_t bb = gbit + r * a.B + a.phi[(uint64_t)d * a.R + r];
-                            if ((bb >> 6) != cur) {
-                                if (bits) atomicOr(idx64 + cur, (unsigned long long)bits);
-                                cur = bb >> 6;
-                                bits = 0;
-                            }
-                            bits |= 1ull << (bb & 63);
-                        }
-                        if (bits) atomicOr(idx64 + cur, (unsigned long long)bits);
-                    }
-                }
+                set((uint32_t)(a.m_pow2 ? (h & (a.m - 1)) : (h % a.m)), d);
             }
         }
     }
+}
+
+// The documents' patterns (RecordSetter KIND 1 and 2): word w of document d's
+// group bits.
+__global__ void k_patterns(unsigned long long *pattern, const uint32_t *phi, uint32_t K, uint32_t R, uint32_t B,
+                           uint32_t Gw) {
+    const uint32_t words = Gw > 1 ? Gw / 2 : 1;
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (uint64_t)K * words) return;
+    const uint64_t d = i / words;
+    const uint32_t w = (uint32_t)(i % words);
+    unsigned long long v = 0;
+    for (uint32_t r = 0; r < R; ++r) {
+        const uint32_t bb = r * B + phi[d * R + r];
+        if ((bb >> 6) == w) v |= 1ull << (bb & 63);
+    }
+    if (Gw > 1) pattern[i] = v;
+    else reinterpret_cast<uint32_t *>(pattern)[i] = (uint32_t)v;
 }
 
 // --------------------------------------------------------------------- fold
@@ -350,21 +331,20 @@ int blocks_per_sm(KernelT kernel, int threads) {
     return n;
 }
 
+template <int ETA, int KIND>
+cudaError_t launch_insert_k(const InsertArgs &a, int sm_count, cudaStream_t s) {
+    static int occ = blocks_per_sm(k_insert<ETA, KIND>, INSERT_THREADS);
+    k_insert<ETA, KIND><<<sm_count * occ, INSERT_THREADS, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <int ETA>
 cudaError_t launch_insert_t(const InsertArgs &a, int sm_count, cudaStream_t s) {
-    // 64-bit words need the index (m * Gw words) to end on a 64-bit boundary
-    const int mode = a.mode == 2 && (a.m * a.Gw) % 2 != 0 ? 1 : (int)a.mode;
-    if (mode == 1) {
-        static int occ = blocks_per_sm(k_insert<ETA, 1>, INSERT_THREADS);
-        k_insert<ETA, 1><<<sm_count * occ, INSERT_THREADS, 0, s>>>(a);
-    } else if (mode == 2) {
-        static int occ = blocks_per_sm(k_insert<ETA, 2>, INSERT_THREADS);
-        k_insert<ETA, 2><<<sm_count * occ, INSERT_THREADS, 0, s>>>(a);
-    } else {
-        static int occ = blocks_per_sm(k_insert<ETA, 0>, INSERT_THREADS);
-        k_insert<ETA, 0><<<sm_count * occ, INSERT_THREADS, 0, s>>>(a);
+    switch (a.kind) {
+        case 0: return launch_insert_k<ETA, 0>(a, sm_count, s);
+        case 1: return launch_insert_k<ETA, 1>(a, sm_count, s);
+        default: return launch_insert_k<ETA, 2>(a, sm_count, s);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -416,6 +396,17 @@ cudaError_t launch_fold(const uint32_t *old_index, uint32_t old_gw, uint32_t *ne
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_fold_docbits<<<sm_count * 4, 256, 0, s>>>(old_db, new_db, B, R, W);
+    return cudaGetLastError();
+}
+
+uint64_t pattern_bytes(const Geometry &g) {
+    if (g.Gw == 1) return (uint64_t)g.K * 4;
+    return g.Gw <= g.R ? (uint64_t)g.K * (g.Gw / 2) * 8 : 0;
+}
+
+cudaError_t launch_patterns(const Geometry &g, unsigned long long *pattern, const uint32_t *phi, cudaStream_t s) {
+    const uint64_t n = (uint64_t)g.K * (g.Gw > 1 ? g.Gw / 2 : 1);
+    k_patterns<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pattern, phi, g.K, g.R, g.B, g.Gw);
     return cudaGetLastError();
 }
 

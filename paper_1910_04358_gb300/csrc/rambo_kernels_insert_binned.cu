@@ -13,12 +13,12 @@
 //   apply    a persistent grid claims units of records in bin order, so all
 //            CTAs work inside one or two regions at a time and the regions
 //            stay in L2 while their records set bit r*B + phi_r(d) of group
-//            h_j(x) for every r (repetitions sharing a 64-bit word merged
-//            into one atomicOr, as the direct insert does).
+//            h_j(x) for every r (RecordSetter, as in the direct insert).
 // Records past a bin's capacity set their bits during the scatter pass.  OR
 // is commutative and idempotent, so the index is bit-identical to the
 // direct insert's whatever the order.
 #include "rambo_insert_binned.cuh"
+#include "rambo_insert_common.cuh"
 
 namespace rgpu {
 namespace {
@@ -27,29 +27,9 @@ constexpr int IB_THREADS = 256;
 constexpr uint32_t IB_UNIT = 2048;  // records per unit of the apply pass
 constexpr uint32_t NO_RANK = 0xffffffffu;
 
-// Sets the bits of one record: bit r*B + phi_r(d) of position group p for
-// every repetition r; `wide` merges repetitions that share a 64-bit word.
-__device__ __forceinline__ void or_record(const InsertArgs &a, uint64_t p, uint32_t d, bool wide) {
-    const uint64_t gbit = p * a.Gw * 32;  // first bit of the group
-    if (wide) {
-        unsigned long long *idx64 = reinterpret_cast<unsigned long long *>(a.index);
-        uint64_t cur = ~0ULL, bits = 0;
-        for (uint32_t r = 0; r < a.R; ++r) {
-            const uint64_t bb = gbit + r * a.B + __ldg(a.phi + (uint64_t)d * a.R + r);
-            if ((bb >> 6) != cur) {
-                if (bits) atomicOr(idx64 + cur, (unsigned long long)bits);
-                cur = bb >> 6;
-                bits = 0;
-            }
-            bits |= 1ull << (bb & 63);
-        }
-        if (bits) atomicOr(idx64 + cur, (unsigned long long)bits);
-    } else {
-        for (uint32_t r = 0; r < a.R; ++r) {
-            const uint64_t bb = gbit + r * a.B + __ldg(a.phi + (uint64_t)d * a.R + r);
-            atomicOr(a.index + (bb >> 5), 1u << (bb & 31));
-        }
-    }
+__device__ __forceinline__ uint32_t record_group(unsigned long long rec) { return (uint32_t)(rec >> IB_DOC_BITS); }
+__device__ __forceinline__ uint32_t record_doc(unsigned long long rec) {
+    return (uint32_t)(rec & ((1u << IB_DOC_BITS) - 1));
 }
 
 // Scatter pass over [f0, f1) of the flat k-mer index: each CTA takes a
@@ -117,9 +97,9 @@ __device__ uint32_t ib_block_scan(uint32_t *v, uint32_t n) {
     return total;
 }
 
-template <int ETA, bool SORTED>
+template <int ETA, bool SORTED, int KIND>
 __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_scatter(InsertArgs a, BinnedInsert b, uint64_t f0,
-                                                                   uint64_t f1, bool wide) {
+                                                                   uint64_t f1) {
     constexpr uint32_t TK = IB_TILE_RECORDS / ETA;  // k-mers per tile
     constexpr uint32_t KPT = TK / IB_THREADS;       // k-mers per thread per tile
     static_assert(KPT * IB_THREADS * ETA == IB_TILE_RECORDS, "tile of whole k-mer rounds");
@@ -152,6 +132,7 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_scatter(InsertArgs a,
         else hi = mid;
     }
     const uint64_t item_first = lo;
+    RecordSetter<KIND> set(a, threadIdx.x & 31);
 
     for (uint32_t jb = 0; jb < a.eta; jb += ETA) {
         uint64_t item = item_first;
@@ -209,22 +190,32 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_scatter(InsertArgs a,
                 }
                 __syncthreads();
                 // 4. the records, or their bits when the bin is full
-                for (uint32_t i = threadIdx.x; i < total; i += IB_THREADS) {
-                    const unsigned long long rec = s_sorted[i];
-                    const uint32_t bin = (uint32_t)((rec >> IB_DOC_BITS) >> b.rshift);
-                    const uint64_t at = (uint64_t)s_base[bin] + (i - s_pre[bin]);
-                    if (at < b.cap) b.buf[(uint64_t)bin * b.cap + at] = rec;
-                    else or_record(a, rec >> IB_DOC_BITS, (uint32_t)(rec & ((1u << IB_DOC_BITS) - 1)), wide);
+                for (uint32_t i0 = 0; i0 < total; i0 += IB_THREADS) {
+                    const uint32_t i = i0 + threadIdx.x;
+                    unsigned long long rec = 0;
+                    bool full = false;
+                    if (i < total) {
+                        rec = s_sorted[i];
+                        const uint32_t bin = (uint32_t)((rec >> IB_DOC_BITS) >> b.rshift);
+                        const uint64_t at = (uint64_t)s_base[bin] + (i - s_pre[bin]);
+                        full = at >= b.cap;
+                        if (!full) b.buf[(uint64_t)bin * b.cap + at] = rec;
+                    }
+                    set(record_group(rec), full ? record_doc(rec) : NO_DOC);
                 }
             } else {
                 // 3. the records in slot order, or their bits when the bin is full
                 for (uint32_t slot = threadIdx.x; slot < IB_TILE_RECORDS; slot += IB_THREADS) {
                     const uint32_t bin = s_bin[slot];
-                    if (bin == NO_RANK) continue;
-                    const unsigned long long rec = s_rec[slot];
-                    const uint64_t at = (uint64_t)s_base[bin] + s_rank[slot];
-                    if (at < b.cap) b.buf[(uint64_t)bin * b.cap + at] = rec;
-                    else or_record(a, rec >> IB_DOC_BITS, (uint32_t)(rec & ((1u << IB_DOC_BITS) - 1)), wide);
+                    unsigned long long rec = 0;
+                    bool full = false;
+                    if (bin != NO_RANK) {
+                        rec = s_rec[slot];
+                        const uint64_t at = (uint64_t)s_base[bin] + s_rank[slot];
+                        full = at >= b.cap;
+                        if (!full) b.buf[(uint64_t)bin * b.cap + at] = rec;
+                    }
+                    set(record_group(rec), full ? record_doc(rec) : NO_DOC);
                 }
             }
             __syncthreads();  // the staging is the next tile's
@@ -233,7 +224,8 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_scatter(InsertArgs a,
 }
 
 // Apply pass: units of IB_UNIT records, claimed in bin order.
-__global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, BinnedInsert b, bool wide) {
+template <int KIND>
+__global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, BinnedInsert b) {
     __shared__ uint32_t s_pre[IB_MAX_BINS + 1];  // units before bin i
     __shared__ uint32_t s_unit;
     // units per bin, then their exclusive prefix (warp 0: lane l sums bins
@@ -264,6 +256,7 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, B
     }
     __syncthreads();
     const uint32_t units = s_pre[b.nbins];
+    RecordSetter<KIND> set(a, threadIdx.x & 31);
     uint32_t *claim = b.count + IB_MAX_BINS;
     while (true) {
         if (threadIdx.x == 0) s_unit = atomicAdd(claim, 1u);
@@ -281,13 +274,17 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, B
         const uint64_t n = b.count[lo] < b.cap ? b.count[lo] : b.cap;
         const uint64_t r0 = (uint64_t)(u - s_pre[lo]) * IB_UNIT;
         const unsigned long long *src = b.buf + (uint64_t)lo * b.cap;
-        for (uint32_t k = threadIdx.x; k < IB_UNIT; k += IB_THREADS) {
-            const uint64_t r = r0 + k;
-            if (r < n) {
-                const unsigned long long rec = __ldcs(src + r);  // read once: do not keep in L2
-                or_record(a, rec >> IB_DOC_BITS, (uint32_t)(rec & ((1u << IB_DOC_BITS) - 1)), wide);
-            }
+        // every thread's records of the unit, loaded before any is set (read
+        // once: not kept in L2)
+        unsigned long long rec[IB_UNIT / IB_THREADS];
+#pragma unroll
+        for (uint32_t k = 0; k < IB_UNIT / IB_THREADS; ++k) {
+            const uint64_t r = r0 + k * IB_THREADS + threadIdx.x;
+            rec[k] = r < n ? __ldcs(src + r) : ~0ull;
         }
+#pragma unroll
+        for (uint32_t k = 0; k < IB_UNIT / IB_THREADS; ++k)
+            set(record_group(rec[k]), r0 + k * IB_THREADS + threadIdx.x < n ? record_doc(rec[k]) : NO_DOC);
     }
 }
 
@@ -299,32 +296,42 @@ int ib_blocks_per_sm(KernelT kernel) {
     return n;
 }
 
-template <int ETA, bool SORTED>
-cudaError_t launch_scatter_t(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1, bool wide,
-                             int sm_count, cudaStream_t s) {
+template <int ETA, bool SORTED, int KIND>
+cudaError_t launch_scatter_t(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1, int sm_count,
+                             cudaStream_t s) {
     constexpr size_t smem = scatter_smem<SORTED>();
-    static int occ = [] {
+    const auto kernel = k_insert_bin_scatter<ETA, SORTED, KIND>;
+    static int occ = [kernel] {
         int n = 0;
-        if (cudaFuncSetAttribute(k_insert_bin_scatter<ETA, SORTED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_insert_bin_scatter<ETA, SORTED>, IB_THREADS,
-                                                          smem) != cudaSuccess ||
-            n < 1)
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, IB_THREADS, smem) != cudaSuccess || n < 1)
             n = 1;
         return n;
     }();
-    cudaError_t e = cudaFuncSetAttribute(k_insert_bin_scatter<ETA, SORTED>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_insert_bin_scatter<ETA, SORTED><<<sm_count * occ, IB_THREADS, smem, s>>>(a, b, f0, f1, wide);
+    kernel<<<sm_count * occ, IB_THREADS, smem, s>>>(a, b, f0, f1);
     return cudaGetLastError();
 }
 
-template <int ETA>
-cudaError_t launch_scatter(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1, bool wide,
-                           int sm_count, cudaStream_t s) {
-    return b.nbins >= IB_SORT_MIN_BINS ? launch_scatter_t<ETA, true>(a, b, f0, f1, wide, sm_count, s)
-                                       : launch_scatter_t<ETA, false>(a, b, f0, f1, wide, sm_count, s);
+template <int ETA, int KIND>
+cudaError_t launch_scatter(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1, int sm_count,
+                           cudaStream_t s) {
+    return b.nbins >= IB_SORT_MIN_BINS ? launch_scatter_t<ETA, true, KIND>(a, b, f0, f1, sm_count, s)
+                                       : launch_scatter_t<ETA, false, KIND>(a, b, f0, f1, sm_count, s);
+}
+
+template <int KIND>
+cudaError_t launch_binned_k(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1, int sm_count,
+                            cudaStream_t s) {
+    cudaError_t e;
+    if (a.eta == 1) e = launch_scatter<1, KIND>(a, b, f0, f1, sm_count, s);
+    else if (a.eta == 2) e = launch_scatter<2, KIND>(a, b, f0, f1, sm_count, s);
+    else e = launch_scatter<4, KIND>(a, b, f0, f1, sm_count, s);
+    if (e != cudaSuccess) return e;
+    static int occ = ib_blocks_per_sm(k_insert_bin_apply<KIND>);
+    k_insert_bin_apply<KIND><<<sm_count * occ, IB_THREADS, 0, s>>>(a, b);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -342,16 +349,11 @@ uint32_t binned_insert_bins(uint64_t m, uint32_t group_bytes, uint32_t K, uint64
 
 cudaError_t launch_insert_binned(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1,
                                  int sm_count, cudaStream_t s) {
-    // 64-bit words need the index (m * Gw words) to end on a 64-bit boundary
-    const bool wide = (a.m * a.Gw) % 2 == 0;
-    cudaError_t e;
-    if (a.eta == 1) e = launch_scatter<1>(a, b, f0, f1, wide, sm_count, s);
-    else if (a.eta == 2) e = launch_scatter<2>(a, b, f0, f1, wide, sm_count, s);
-    else e = launch_scatter<4>(a, b, f0, f1, wide, sm_count, s);
-    if (e != cudaSuccess) return e;
-    static int occ = ib_blocks_per_sm(k_insert_bin_apply);
-    k_insert_bin_apply<<<sm_count * occ, IB_THREADS, 0, s>>>(a, b, wide);
-    return cudaGetLastError();
+    switch (a.kind) {
+        case 0: return launch_binned_k<0>(a, b, f0, f1, sm_count, s);
+        case 1: return launch_binned_k<1>(a, b, f0, f1, sm_count, s);
+        default: return launch_binned_k<2>(a, b, f0, f1, sm_count, s);
+    }
 }
 
 }  // namespace rgpu
