@@ -653,7 +653,8 @@ int insert_enqueue(rambo_t *h, uint64_t n, const uint32_t *doc_ids, const uint8_
     const uint64_t chunks = (bound + per - 1) / per;
     if (chunks > IB_MAX_CHUNKS) nbins = 0;
     if (nbins) {
-        BinnedInsert b{h->d_bins, h->d_bin_count, h->bins_records / nbins, nbins, rshift};
+        // (an even number of slots a bin: the apply pass copies records in pairs)
+        BinnedInsert b{h->d_bins, h->d_bin_count, h->bins_records / nbins & ~1ull, nbins, rshift};
         StageScope sc(h, RAMBO_STAGE_INSERT, s, (int)(2 * chunks));
         for (uint64_t f0 = 0; f0 < bound; f0 += per) {
             RAMBO_TRY(cudaMemsetAsync(h->d_bin_count, 0, (IB_MAX_BINS + 1) * 4, s));

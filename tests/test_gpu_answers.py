@@ -78,3 +78,37 @@ def test_kmer_answers_latch_bad_codes(rambo_lib):
         idx.query_kmers(kmers)
     assert e.value.code == rambo_lib.RAMBO_EINVAL
     idx.query_kmers(kmers[:77])
+
+
+@pytest.mark.parametrize("K,B,R,m,eta", [
+    (60, 9, 3, 3001, 1),          # 4-byte groups: one word per record; odd m
+    (90, 32, 2, 1 << 12, 3),      # 8-byte groups: one 64-bit word per record
+    (200, 31, 4, 1 << 12, 2),     # 16-byte groups: two words per record
+    (120, 40, 3, 1 << 12, 5),     # 16-byte groups: a lane per repetition, eta past one pass
+    (80, 30, 9, 1 << 11, 2),      # 64-byte groups, nine repetitions
+    (50, 3, 40, 1 << 11, 2),      # more repetitions than lanes, groups of few words
+    (40, 70, 33, 1 << 10, 1),     # more repetitions than lanes, a lane per repetition
+])
+def test_insert_record_shapes_match_oracle(rambo_lib, K, B, R, m, eta):
+    # documents shorter and longer than a thread's run of k-mers, empty ones
+    # among them; direct, binned, and binned with bins that overflow
+    p = synth.Params(K=K, B=B, R=R, m=m, eta=eta, k=21, seed=K)
+    rng = np.random.default_rng(K * 3 + R)
+    lens = np.concatenate([[0, 20, 21, 22, 28, 29, 37], rng.integers(21, 400, size=K - 8), [9001]])
+    packed, offs = synth.pack_many([synth.uniform_genome(rng, int(n)) for n in lens])
+    ids = rng.permutation(K).astype(np.uint32)
+    o = oracle.Rambo(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    o.insert_batch(ids, packed, offs)
+    for st in (dict(insert_mode=2), dict(insert_mode=3, bin_region_kib=16),
+               dict(insert_mode=3, bin_region_kib=1, insert_bin_records=4096)):
+        idx = rambo_lib.Index(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+        idx.set_tuning(**st)
+        idx.insert_batch(ids, packed, offs)
+        words = idx.copy_index().view(np.uint32).reshape(m, -1)
+        bits = np.unpackbits(words.view(np.uint8), axis=1, bitorder="little")
+        for r in range(R):
+            for b in range(B):
+                want = np.unpackbits(o.filter_words(r, b).view(np.uint8), bitorder="little")[:m]
+                assert np.array_equal(bits[:, r * B + b], want), (st, r, b)
+        assert not bits[:, R * B:].any()
+        idx.close()
