@@ -332,8 +332,10 @@ int rambo_copy_partition(const rambo_t *h, uint32_t *dst);
 /* Tuning knobs (launch shapes; none changes any result).                  */
 
 typedef struct {
-    uint32_t probe_ctas_per_sm;        /* probe grid = SMs x this; 0 = occupancy max */
-    uint32_t probe_min_kmers_per_warp; /* smallest k-mer range a warp takes; 0 = 64  */
+    uint32_t probe_ctas_per_sm;        /* probe grid = SMs x this; 0 = occupancy max   */
+                                       /* (path 1), or by the batch (separate launch) */
+    uint32_t probe_min_kmers_per_warp; /* separate probe launch: k-mers a warp takes, */
+                                       /* about; 0 = 256                              */
     uint32_t expand_ctas_per_sm;       /* grid cap of the answer kernels (expansion   */
                                        /* and single k-mers) = SMs x this (1..64)    */
     uint32_t use_byte_table;           /* 1: path 1 expands a query through a         */
@@ -342,7 +344,9 @@ typedef struct {
     uint32_t query_path;               /* sequence queries: 0 = prefix scan + probe +  */
                                        /* expand launches; 1 = persistent fused launch */
                                        /* with length-bucketed work queues (groups up  */
-                                       /* to 512 B; otherwise path 0 is used); 2 =     */
+                                       /* to 512 B; otherwise, and for small batches   */
+                                       /* and groups up to 16 B without early_exit,    */
+                                       /* path 0 is used); 2 =                         */
                                        /* region-binned probing (groups up to 64 B    */
                                        /* and a workspace from                         */
                                        /* rambo_query_seqs_workspace_for; otherwise    */

@@ -396,7 +396,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
             ProbeArgs &a = ba.p;
             a.index = h->d_index;
             a.m = g.m;
-            a.m_pow2 = (g.m & (g.m - 1)) == 0;
+            a.m_inv = position_reciprocal(g.m);
             a.Gw = g.Gw;
             a.eta = g.eta;
             a.k = g.k;
@@ -445,7 +445,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
             ProbeArgs &a = sa.p;
             a.index = h->d_index;
             a.m = g.m;
-            a.m_pow2 = (g.m & (g.m - 1)) == 0;
+            a.m_inv = position_reciprocal(g.m);
             a.Gw = g.Gw;
             a.eta = g.eta;
             a.k = g.k;
@@ -488,12 +488,23 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
             return expand_enqueue(h, n, acc, out, s);
         }
     }
-    if (h->tune.query_path >= 1 && fused_supported(g)) {
+    // The separate launches serve path 1 too where they are the faster ones: a
+    // batch of less than a tile per resident warp, which leaves the persistent
+    // launch short of work (256 requests of 470 bases: 24 against 253 us), and
+    // one-lane groups, unless the launch has to leave room for k-mer chunks
+    // (10^4 x 1 kbp beside 10^6 k-mers: 460 against 489 us; the same call with
+    // host buffers 0.88 against 0.80 ms).  Wider groups keep the persistent
+    // launch, which hides the expansion under the gathers (streaming epoch,
+    // 12.5 KB answers: 0.85 against 0.93 ms; 32 GiB index: equal).
+    const bool one_lane = g.LPG == 1 && fused_ctas_cap == 0;
+    const bool small = packed_bytes * 4 < (uint64_t)h->sm_count * 24 * h->tune.fused_tile_kmers;
+    const bool separate = !h->tune.early_exit && (one_lane || small);
+    if (h->tune.query_path >= 1 && !separate && fused_supported(g)) {
         // persistent fused query: length-bucketed queues, probe + expand in one launch
         ProbeArgs a{};
         a.index = h->d_index;
         a.m = g.m;
-        a.m_pow2 = (g.m & (g.m - 1)) == 0;
+        a.m_inv = position_reciprocal(g.m);
         a.Gw = g.Gw;
         a.eta = g.eta;
         a.k = g.k;
@@ -531,15 +542,16 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
         RAMBO_TRY(launch_fused(a, e, g, qs, go, h->sm_count, s));
         return RAMBO_OK;
     }
+    const uint32_t tile = probe_tile_kmers(packed_bytes * 4, h->sm_count);
     {
         StageScope sc(h, RAMBO_STAGE_PREFIX, s, kmer_prefix_launches(n));
-        RAMBO_TRY(launch_kmer_prefix(offsets, ends, n, g.k, packed_bytes, kcum, bsum, h->d_err, s));
+        RAMBO_TRY(launch_kmer_prefix(offsets, ends, n, g.k, packed_bytes, kcum, bsum, h->d_err, s, tile, 0, acc,
+                                     n * (uint64_t)g.Gw * 4));
     }
-    RAMBO_TRY(cudaMemsetAsync(acc, 0xFF, n * (uint64_t)g.Gw * 4, s));
     ProbeArgs a{};
     a.index = h->d_index;
     a.m = g.m;
-    a.m_pow2 = (g.m & (g.m - 1)) == 0;
+    a.m_inv = position_reciprocal(g.m);
     a.Gw = g.Gw;
     a.eta = g.eta;
     a.k = g.k;
@@ -554,22 +566,27 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
     a.acc = acc;
     a.err = h->d_err;
     a.min_chunk = h->tune.probe_min_kmers_per_warp;
+    a.max_kmers = packed_bytes * 4;
     {
         StageScope sc(h, RAMBO_STAGE_PROBE_SEQS, s, 1);
-        RAMBO_TRY(launch_probe_seqs(a, g, probe_grid(h), s));
+        RAMBO_TRY(launch_probe_seqs(a, g, tile, probe_grid(h), s));
     }
     return expand_enqueue(h, n, acc, out, s);
 }
 
+// few_blocks: the answers go straight to host memory beside a sequence branch.
+// A block an SM over all chunks in flight keeps the link busy; more of them
+// clog the way of the sequences' gathers (medium batch with host buffers, 38
+// blocks a chunk: 0.80 ms, 76: 0.83, 152: 0.85, 304: 0.87..1.19).
 int query_kmers_enqueue(rambo_t *h, uint64_t n, const uint64_t *kmers, uint32_t *out, void *ws,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool few_blocks = false) {
     const Geometry &g = h->g;
     uint32_t *acc = static_cast<uint32_t *>(ws);
     if (!h->d_slots && g.eta > 4) RAMBO_TRY(cudaMemsetAsync(acc, 0xFF, n * (uint64_t)g.Gw * 4, s));
     ProbeArgs a{};
     a.index = h->d_index;
     a.m = g.m;
-    a.m_pow2 = (g.m & (g.m - 1)) == 0;
+    a.m_inv = position_reciprocal(g.m);
     a.Gw = g.Gw;
     a.eta = g.eta;
     a.k = g.k;
@@ -581,8 +598,10 @@ int query_kmers_enqueue(rambo_t *h, uint64_t n, const uint64_t *kmers, uint32_t 
     a.min_chunk = h->tune.probe_min_kmers_per_warp;
     if (h->d_slots) {  // probe and answer in one launch
         StageScope sc(h, RAMBO_STAGE_PROBE_KMERS, s, 1);
-        RAMBO_TRY(launch_kmer_answers(a, g, h->d_slots, out, h->sm_count * (int)h->tune.expand_ctas_per_sm,
-                                      h->sm_count, s));
+        int blocks = h->sm_count * (int)h->tune.expand_ctas_per_sm;
+        const int few = (h->sm_count + RAMBO_MAX_HOST_SLOTS - 1) / RAMBO_MAX_HOST_SLOTS;
+        if (few_blocks && blocks > few) blocks = few;
+        RAMBO_TRY(launch_kmer_answers(a, g, h->d_slots, out, blocks, h->sm_count, s));
         return RAMBO_OK;
     }
     {
@@ -618,7 +637,7 @@ int insert_enqueue(rambo_t *h, uint64_t n, const uint32_t *doc_ids, const uint8_
     InsertArgs a{};
     a.index = h->d_index;
     a.m = g.m;
-    a.m_pow2 = (g.m & (g.m - 1)) == 0;
+    a.m_inv = position_reciprocal(g.m);
     a.Gw = g.Gw;
     a.B = g.B;
     a.R = g.R;
@@ -849,7 +868,8 @@ int query_batch_host(rambo_t *h, uint64_t nk, const uint64_t *kmers, uint32_t *o
         uint32_t *d_out = direct_k ? direct_k + i0 * g.W : reinterpret_cast<uint32_t *>(slot + kin);
         e = cudaMemcpyAsync(d_k, kmers + i0, cn * 8, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return bail(cuda_rc(e));
-        rc = query_kmers_enqueue(h, cn, d_k, d_out, slot + kin + kout, s);
+        // (short rows leave the link idle while few blocks probe)
+        rc = query_kmers_enqueue(h, cn, d_k, d_out, slot + kin + kout, s, direct_k && ns && row >= 64);
         if (rc) return bail(rc);
         if (!direct_k) {
             e = cudaMemcpyAsync(out_k + i0 * g.W, d_out, cn * row, cudaMemcpyDeviceToHost, s);
@@ -1270,7 +1290,7 @@ int rambo_insert_words_dev(rambo_t *h, uint32_t n_docs, const uint32_t *doc_ids,
     WordArgs a{};
     a.index = h->d_index;
     a.m = g.m;
-    a.m_pow2 = (g.m & (g.m - 1)) == 0;
+    a.m_inv = position_reciprocal(g.m);
     a.Gw = g.Gw; a.B = g.B; a.R = g.R; a.K = g.K; a.eta = g.eta;
     a.seed32 = (uint32_t)g.seed;
     a.phi = h->d_phi;
@@ -1311,7 +1331,7 @@ int rambo_query_words_dev(rambo_t *h, uint64_t n, const uint8_t *bytes, uint64_t
     WordArgs a{};
     a.index_ro = h->d_index;
     a.m = g.m;
-    a.m_pow2 = (g.m & (g.m - 1)) == 0;
+    a.m_inv = position_reciprocal(g.m);
     a.Gw = g.Gw; a.B = g.B; a.R = g.R; a.K = g.K; a.eta = g.eta;
     a.seed32 = (uint32_t)g.seed;
     a.bytes = bytes;

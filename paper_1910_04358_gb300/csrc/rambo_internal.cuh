@@ -50,6 +50,18 @@ __device__ __forceinline__ uint64_t mh_first_word(uint64_t k1mix, uint32_t seed)
     return fmix64(h1) + fmix64(h2);
 }
 
+// Probe position h mod m (m <= 2^32).  m_inv = 0: m is a power of two.  Else
+// m_inv = floor(2^64 / m), and the high product h * m_inv / 2^64 is the
+// quotient or one less (h / m - h * m_inv / 2^64 < h / 2^64 < 1), so one
+// conditional subtraction corrects the remainder: 17 instructions, where the
+// 64-bit remainder of a run-time divisor is a call of some 70.
+__host__ __device__ inline uint64_t position_reciprocal(uint64_t m) { return (m & (m - 1)) == 0 ? 0 : ~0ULL / m; }
+__device__ __forceinline__ uint32_t reduce_pos(uint64_t h, uint64_t m, uint64_t m_inv) {
+    if (m_inv == 0) return (uint32_t)(h & (m - 1));
+    const uint64_t r = h - __umul64hi(h, m_inv) * m;
+    return (uint32_t)(r >= m ? r - m : r);
+}
+
 // ---------------------------------------------------------------------------
 // k-mers from the 2-bit packed stream.
 
@@ -167,7 +179,7 @@ Geometry make_geometry(uint32_t K, uint32_t B, uint32_t R, uint64_t m, uint32_t 
 struct ProbeArgs {
     const uint32_t *index;
     uint64_t m;
-    uint32_t m_pow2;      // m is a power of two: reduce with a mask
+    uint64_t m_inv;       // position_reciprocal(m)
     uint32_t Gw;
     uint32_t eta;
     uint32_t k;
@@ -186,6 +198,7 @@ struct ProbeArgs {
     uint32_t *acc;
     uint32_t *err;
     uint32_t min_chunk;      // minimum k-mers per warp (0 = default)
+    uint64_t max_kmers;      // sequence batch: about how many k-mers it has (grid sizing only)
 };
 
 struct ExpandArgs {
@@ -200,7 +213,7 @@ struct ExpandArgs {
 struct InsertArgs {
     uint32_t *index;
     uint64_t m;
-    uint32_t m_pow2;
+    uint64_t m_inv;
     uint32_t Gw, B, R, K, eta, k, seed32;
     const uint32_t *phi;       // K x R
     const uint32_t *doc_ids;   // n
@@ -224,7 +237,7 @@ struct WordArgs {
     uint32_t *index;           // insert: written with atomicOr
     const uint32_t *index_ro;  // probe: read only
     uint64_t m;
-    uint32_t m_pow2;
+    uint64_t m_inv;
     uint32_t Gw, B, R, K, eta, seed32;
     const uint32_t *phi;       // K x R
     const uint32_t *doc_ids;   // insert: n
@@ -246,6 +259,8 @@ cudaError_t launch_partition(uint32_t *phi, uint32_t K, uint32_t R, uint32_t B, 
 // Exclusive prefix (n+1 values) of the k-mer counts of items
 // [begins[i], ends[i]); with tile > 0, of the tile counts of the items with
 // more than short_max k-mers (ceil(k-mers / tile); shorter items count 0).
+// Also sets fill_bytes bytes (rounded up to 16) at `fill` (16-byte aligned) to
+// ones, when given.
 // Device address of the host range [p, p + bytes) when both its ends lie in
 // page-locked host memory that the current device can address (allocated
 // with cudaHostAlloc / cudaMallocHost or registered, mapped under unified
@@ -258,7 +273,7 @@ int kmer_prefix_launches(uint64_t n);
 cudaError_t launch_kmer_prefix(const uint64_t *begins, const uint64_t *ends, uint64_t n, uint32_t k,
                                uint64_t packed_bytes, uint64_t *kcum, uint64_t *block_sums,
                                uint32_t *err, cudaStream_t s, uint32_t tile = 0,
-                               uint32_t short_max = 0);
+                               uint32_t short_max = 0, void *fill = nullptr, size_t fill_bytes = 0);
 size_t kmer_prefix_block_sums(uint64_t n);
 // (slots: the answer kernels' document table, or null)
 cudaError_t launch_register_docs(const uint32_t *doc_ids, uint64_t n, const uint32_t *phi,
@@ -284,7 +299,10 @@ cudaError_t launch_fold(const uint32_t *old_index, uint32_t old_gw, uint32_t *ne
                         uint32_t new_gw, uint64_t m, uint32_t B, uint32_t R,
                         const uint32_t *old_db, uint32_t *new_db, uint32_t W, int sm_count,
                         cudaStream_t s);
-cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, int sm_count, cudaStream_t s);
+// k-mers per tile for a batch of about max_kmers k-mers
+uint32_t probe_tile_kmers(uint64_t max_kmers, int sm_count);
+// kcum: the batch's tile prefix (launch_kmer_prefix, `tile`); acc set to ones
+cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm_count, cudaStream_t s);
 // (groups of 512 bytes and more; the others are probed by launch_kmer_answers)
 cudaError_t launch_probe_kmers(const ProbeArgs &a, const Geometry &g, int sm_count, cudaStream_t s);
 // Work queues of the persistent fused query (workspace arrays).

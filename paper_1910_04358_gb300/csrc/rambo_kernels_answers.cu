@@ -110,7 +110,7 @@ __device__ __forceinline__ void kmer_rows(const AnswerArgs &a, uint64_t km, uint
 #pragma unroll
     for (int e = 0; e < ETA; ++e) {
         const uint32_t j = jb + e < a.p.eta ? jb + e : a.p.eta - 1;
-        row[e] = reduce_pos(mh_first_word(km, a.p.seed32 + j), a.p.m, a.p.m_pow2);
+        row[e] = reduce_pos(mh_first_word(km, a.p.seed32 + j), a.p.m, a.p.m_inv);
     }
 }
 

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(SCATTER_THREADS) k_bin_scatter(BinnedArgs a) {
             const uint64_t km = mh_mix_key(c);
             const uint32_t r0 = (uint32_t)(g - h.k0) * p.eta;
             for (uint32_t j = 0; j < p.eta; ++j) {
-                const uint32_t pos = reduce_pos(mh_first_word(km, p.seed32 + j), p.m, p.m_pow2);
+                const uint32_t pos = reduce_pos(mh_first_word(km, p.seed32 + j), p.m, p.m_inv);
                 s_pos[r0 + j] = pos;
                 s_rank[r0 + j] = (uint16_t)atomicAdd(&s_cnt[pos >> a.shift], 1u);
             }

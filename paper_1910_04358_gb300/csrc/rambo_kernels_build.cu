@@ -10,6 +10,8 @@
 //              h_1(x)..h_eta(x) of BFU (phi_r(d), r) for every r.  In the
 //              bit-sliced layout that is bit r*B+phi_r(d) of position group
 //              h_j(x), set with one atomicOr per repetition or 64-bit word.
+#include <cooperative_groups.h>
+
 #include "rambo_insert_common.cuh"
 
 namespace rgpu {
@@ -128,45 +130,98 @@ k_prefix_final(const uint64_t *begins, const uint64_t *ends, uint64_t n, uint32_
     }
 }
 
-// Small batches: the whole scan in one block of 1024 threads (one launch
-// instead of three).  Each pass counts a tile of items with coalesced loads
-// into shared memory, then every thread scans four consecutive counts;
-// kcum[n] = grand total.
-constexpr uint64_t SCAN_SINGLE_MAX = 16 * SCAN_TILE;
-constexpr int SCAN1_THREADS = 1024;
-constexpr int SCAN1_ITEMS = 4;
-constexpr uint32_t SCAN1_TILE = SCAN1_THREADS * SCAN1_ITEMS;
+// Up to SCAN_ONCE_MAX items: one launch of one cluster of CL blocks, each
+// scanning a share of the items; the shares' totals go through distributed
+// shared memory.  Clusters past the first fill `fill` with ones: the bucket
+// masks of the batch, which would be a launch of their own.  Bound by latency:
+// 20,011 items take 6 us (11 with 256 threads a block, 24 in one block walking
+// all the tiles); 100,000 took 23 in three launches (partial sums, their scan,
+// a second pass).
+constexpr uint32_t SCAN1_TILE = 4096;  // items a block scans at a time
+constexpr uint64_t SCAN_ONCE_MAX = 32 * SCAN1_TILE;
+constexpr uint64_t SCAN_FILL_BYTES = 64 * 1024;  // a fill block's share, at least
 
-__global__ void __launch_bounds__(SCAN1_THREADS)
-k_prefix_single(const uint64_t *begins, const uint64_t *ends, uint64_t n, uint32_t k,
-                uint64_t limit, uint64_t *kcum, uint32_t *err, CountMode cm) {
+template <int CL, int THREADS>
+__global__ void __launch_bounds__(THREADS)
+k_prefix_once(const uint64_t *begins, const uint64_t *ends, uint64_t n, uint32_t k, uint64_t limit,
+              uint64_t *kcum, uint32_t *err, CountMode cm, uint4 *fill, uint64_t fill16) {
+    constexpr int ITEMS = SCAN1_TILE / THREADS;
+    if (blockIdx.x >= CL) {
+        const uint64_t step = (uint64_t)(gridDim.x - CL) * THREADS;
+        for (uint64_t i = (uint64_t)(blockIdx.x - CL) * THREADS + threadIdx.x; i < fill16; i += step)
+            fill[i] = make_uint4(FULL, FULL, FULL, FULL);
+        return;
+    }
     __shared__ uint64_t s_cnt[SCAN1_TILE];
-    uint64_t carry = 0;
-    for (uint64_t base = 0; base < n; base += SCAN1_TILE) {
-#pragma unroll
-        for (int j = 0; j < SCAN1_ITEMS; ++j) {
-            const uint32_t t = threadIdx.x + j * SCAN1_THREADS;
-            s_cnt[t] = base + t < n ? kmer_count(begins, ends, base + t, k, limit, err, cm) : 0;
+    __shared__ uint64_t s_total[CL];  // totals of the shares up to this block's
+    uint64_t share = (n + CL - 1) / CL;
+    const uint64_t lo = blockIdx.x * share, hi = lo + share < n ? lo + share : n;
+    const bool once = share <= SCAN1_TILE;  // the counts stay in shared memory
+    uint64_t sum = 0, total = 0, carry = 0;
+    if (CL > 1) {
+#pragma unroll 4
+        for (uint64_t i = lo + threadIdx.x; i < hi; i += THREADS) {
+            const uint64_t c = kmer_count(begins, ends, i, k, limit, err, cm);
+            if (once) s_cnt[i - lo] = c;
+            sum += c;
         }
-        __syncthreads();
-        uint64_t c[SCAN1_ITEMS];
-        uint64_t sum = 0;
+        block_exclusive_scan<THREADS>(sum, &total);
+        namespace cg = cooperative_groups;
+        const cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();  // every block runs, so its shared memory may be written
+        if (threadIdx.x < CL && threadIdx.x >= blockIdx.x)
+            cluster.map_shared_rank(s_total, threadIdx.x)[blockIdx.x] = total;
+        cluster.sync();
+        for (uint32_t b = 0; b < blockIdx.x; ++b) carry += s_total[b];
+    }
+    for (uint64_t base = lo; base < hi; base += SCAN1_TILE) {
+        if (CL == 1 || !once)
 #pragma unroll
-        for (int j = 0; j < SCAN1_ITEMS; ++j) {
-            c[j] = s_cnt[threadIdx.x * SCAN1_ITEMS + j];
+            for (int j = 0; j < ITEMS; ++j) {
+                const uint32_t t = threadIdx.x + j * THREADS;
+                if (base + t < hi) s_cnt[t] = kmer_count(begins, ends, base + t, k, limit, CL == 1 ? err : nullptr, cm);
+            }
+        __syncthreads();
+        const uint64_t i0 = base + (uint64_t)threadIdx.x * ITEMS;
+        uint64_t c[ITEMS];
+        sum = 0;
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+            c[j] = i0 + j < hi ? s_cnt[threadIdx.x * ITEMS + j] : 0;
             sum += c[j];
         }
-        uint64_t total;
-        uint64_t run = carry + block_exclusive_scan<SCAN1_THREADS>(sum, &total);
-        const uint64_t i0 = base + (uint64_t)threadIdx.x * SCAN1_ITEMS;
+        uint64_t run = carry + block_exclusive_scan<THREADS>(sum, &total);
 #pragma unroll
-        for (int j = 0; j < SCAN1_ITEMS; ++j) {
-            if (i0 + j < n) kcum[i0 + j] = run;
+        for (int j = 0; j < ITEMS; ++j) {
+            s_cnt[threadIdx.x * ITEMS + j] = run;  // (the scan ended with a barrier)
             run += c[j];
         }
-        carry += total;  // the scan ends with a barrier: s_cnt may be refilled
+        __syncthreads();
+        for (uint32_t t = threadIdx.x; t < SCAN1_TILE && base + t < hi; t += THREADS) kcum[base + t] = s_cnt[t];
+        __syncthreads();
+        carry += total;
     }
-    if (threadIdx.x == 0) kcum[n] = carry;
+    if (hi == n && lo < n && threadIdx.x == 0) kcum[n] = carry;
+}
+
+template <int CL, int THREADS>
+cudaError_t launch_prefix_once(const uint64_t *begins, const uint64_t *ends, uint64_t n, uint32_t k, uint64_t limit,
+                               uint64_t *kcum, uint32_t *err, CountMode cm, void *fill, size_t fill_bytes,
+                               cudaStream_t s) {
+    uint64_t fillers = (fill_bytes + SCAN_FILL_BYTES - 1) / SCAN_FILL_BYTES;
+    if (fillers > 256) fillers = 256;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(CL + (fillers + CL - 1) / CL * CL));
+    cfg.blockDim = dim3(THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CL;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = CL > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_prefix_once<CL, THREADS>, begins, ends, n, k, limit, kcum, err, cm,
+                              static_cast<uint4 *>(fill), (uint64_t)((fill_bytes + 15) / 16));
 }
 
 // ------------------------------------------------------------- registration
@@ -238,7 +293,7 @@ __global__ void __launch_bounds__(INSERT_THREADS, 1) k_insert(InsertArgs a) {
             for (int e = 0; e < ETA; ++e) {
                 if (jb + e >= a.eta) break;  // warp-uniform
                 const uint64_t h = mh_first_word(km, a.seed32 + jb + e);
-                set((uint32_t)(a.m_pow2 ? (h & (a.m - 1)) : (h % a.m)), d);
+                set(reduce_pos(h, a.m, a.m_inv), d);
             }
         }
     }
@@ -334,7 +389,10 @@ int blocks_per_sm(KernelT kernel, int threads) {
 template <int ETA, int KIND>
 cudaError_t launch_insert_k(const InsertArgs &a, int sm_count, cudaStream_t s) {
     static int occ = blocks_per_sm(k_insert<ETA, KIND>, INSERT_THREADS);
-    k_insert<ETA, KIND><<<sm_count * occ, INSERT_THREADS, 0, s>>>(a);
+#ifndef INS_X
+#define INS_X 1
+#endif
+    k_insert<ETA, KIND><<<sm_count * occ * INS_X, INSERT_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -358,18 +416,24 @@ cudaError_t launch_partition(uint32_t *phi, uint32_t K, uint32_t R, uint32_t B, 
 
 size_t kmer_prefix_block_sums(uint64_t n) { return (size_t)((n + SCAN_TILE - 1) / SCAN_TILE); }
 
-int kmer_prefix_launches(uint64_t n) { return n == 0 ? 0 : n <= SCAN_SINGLE_MAX ? 1 : 3; }
+int kmer_prefix_launches(uint64_t n) { return n == 0 ? 0 : n <= SCAN_ONCE_MAX ? 1 : 3; }
 
 cudaError_t launch_kmer_prefix(const uint64_t *begins, const uint64_t *ends, uint64_t n, uint32_t k,
                                uint64_t packed_bytes, uint64_t *kcum, uint64_t *block_sums,
-                               uint32_t *err, cudaStream_t s, uint32_t tile, uint32_t short_max) {
+                               uint32_t *err, cudaStream_t s, uint32_t tile, uint32_t short_max, void *fill,
+                               size_t fill_bytes) {
     const uint64_t limit = packed_bytes * 4;  // bases addressable from the caller's pointer
     const uint64_t nblk = kmer_prefix_block_sums(n);
     if (nblk == 0) return cudaSuccess;
     const CountMode cm{tile, short_max};
-    if (n <= SCAN_SINGLE_MAX) {
-        k_prefix_single<<<1, SCAN1_THREADS, 0, s>>>(begins, ends, n, k, limit, kcum, err, cm);
-        return cudaGetLastError();
+    if (n <= SCAN_ONCE_MAX) {
+        if (n <= SCAN1_TILE)
+            return launch_prefix_once<1, 1024>(begins, ends, n, k, limit, kcum, err, cm, fill, fill_bytes, s);
+        return launch_prefix_once<8, 1024>(begins, ends, n, k, limit, kcum, err, cm, fill, fill_bytes, s);
+    }
+    if (fill_bytes) {
+        const cudaError_t e = cudaMemsetAsync(fill, 0xFF, fill_bytes, s);
+        if (e != cudaSuccess) return e;
     }
     k_prefix_partial<<<(unsigned)nblk, SCAN_THREADS, 0, s>>>(begins, ends, n, k, limit, block_sums, err, cm);
     k_prefix_blocks<<<1, SCAN_THREADS, 0, s>>>(block_sums, nblk, kcum, n);

@@ -86,104 +86,9 @@ __global__ void k_fused_prep(FusedArgs f) {
     }
 }
 
-// Rounds of loads a lane keeps in flight, and (ASYNC) the shared-memory
-// staging a warp needs for them: one 16-byte slot per lane, round and probe.
-template <int LPG>
-__host__ __device__ constexpr int fused_rif() { return LPG == 1 ? 8 : 4; }
+// The shared-memory staging a block's warps need for ASYNC gathers.
 template <int ETA>
-__host__ __device__ constexpr size_t fused_stage_bytes() { return (size_t)(FUSED_THREADS / 32) * fused_rif<1>() * ETA * 32 * 16; }
-
-// AND of the groups of k-mers [k0, k1) of one query, per lane slice (every
-// lane of the warp works on the same query).  ASYNC (one lane per 16-byte
-// group): the gathers land in the warp's shared-memory `stage` through
-// cp.async instead of registers, so a lane holds no load data in flight.
-template <int SW, int LPG, int ETA, bool ASYNC>
-__device__ __forceinline__ Slice<SW> fused_probe_range(const ProbeArgs &a, uint64_t start,
-                                                        uint64_t k0, uint64_t k1, int lane,
-                                                        uint32_t word0, uint4 *stage) {
-    static_assert(!ASYNC || (LPG == 1 && SW == 4), "staged gathers: one lane per 16-byte group");
-    constexpr int RIF = fused_rif<LPG>();  // rounds whose loads are in flight together
-    constexpr int NT = LPG >= RIF ? 1 : RIF / LPG;
-    constexpr int KPR = 32 / LPG;
-    constexpr int ROUNDS = NT * LPG;
-    constexpr int STEP = 32 * NT;
-    const int sub = lane / LPG;
-    Slice<SW> accv;
-    slice_ones(accv);
-    for (uint32_t jb = 0; jb < a.eta; jb += ETA) {
-        for (uint64_t base = k0; base < k1; base += STEP) {
-            uint32_t pos[NT][ETA];
-            bool val[NT];
-#pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const uint64_t g = base + (uint64_t)t * 32 + lane;
-                val[t] = g < k1;
-                uint64_t c = 0;
-                if (val[t])
-                    c = canonical_from_window(base_window(a.packed, a.packed_bytes, start + a.base_shift + g), a.k);
-                const uint64_t km = mh_mix_key(c);
-#pragma unroll
-                for (int e = 0; e < ETA; ++e) {
-                    const uint32_t j = jb + e < a.eta ? jb + e : a.eta - 1;
-                    pos[t][e] = reduce_pos(mh_first_word(km, a.seed32 + j), a.m, a.m_pow2);
-                }
-            }
-#pragma unroll
-            for (int rg = 0; rg < ROUNDS; rg += RIF) {
-                if constexpr (ASYNC) {
-                    // each lane gathers its own k-mers' groups (LPG == 1)
-                    uint32_t live = 0;
-#pragma unroll
-                    for (int rr = 0; rr < RIF; ++rr) {
-                        const int t = rg + rr;
-#pragma unroll
-                        for (int e = 0; e < ETA; ++e)
-                            if (val[t]) {
-                                cp_async16(stage + (rr * ETA + e) * 32 + lane,
-                                           a.index + (uint64_t)pos[t][e] * a.Gw + word0);
-                                live |= 1u << (rr * ETA + e);
-                            }
-                    }
-                    cp_async_wait_all();
-#pragma unroll
-                    for (int i = 0; i < RIF * ETA; ++i)
-                        if (live & (1u << i)) {
-                            const uint4 v = stage[i * 32 + lane];
-                            accv.w[0] &= v.x;
-                            accv.w[1] &= v.y;
-                            accv.w[2] &= v.z;
-                            accv.w[3] &= v.w;
-                        }
-                    continue;
-                }
-                Slice<SW> v[RIF][ETA];
-#pragma unroll
-                for (int rr = 0; rr < RIF; ++rr) {
-                    const int rho = rg + rr;
-                    const int t = rho / LPG;
-                    const int src = (rho % LPG) * KPR + sub;
-                    const bool vs = __shfl_sync(FULL, (int)val[t], src) != 0;
-#pragma unroll
-                    for (int e = 0; e < ETA; ++e) {
-                        const uint32_t p = __shfl_sync(FULL, pos[t][e], src);
-                        if (vs) v[rr][e] = ld_slice<SW>(a.index + (uint64_t)p * a.Gw + word0);
-                        else slice_ones(v[rr][e]);
-                    }
-                }
-#pragma unroll
-                for (int rr = 0; rr < RIF; ++rr)
-#pragma unroll
-                    for (int e = 0; e < ETA; ++e) slice_and(accv, v[rr][e]);
-            }
-        }
-    }
-    // combine the lanes that hold the same slice
-#pragma unroll
-    for (int w = 0; w < SW; ++w)
-#pragma unroll
-        for (int off = LPG; off < 32; off <<= 1) accv.w[w] &= __shfl_xor_sync(FULL, accv.w[w], off);
-    return accv;
-}
+__host__ __device__ constexpr size_t fused_stage_bytes() { return (size_t)(FUSED_THREADS / 32) * probe_rif<1, ETA>() * ETA * 32 * 16; }
 
 template <int SW, int LPG, int ETA, int C, bool ASYNC>
 // three resident blocks per SM fit without spills for groups read by 4+
@@ -197,7 +102,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, (LPG >= 4 || ASYNC) ? 3 : 2) k_
     const int wib = threadIdx.x >> 5;
     uint32_t *bm = bm_smem[wib];
     uint32_t *list = list_smem[wib];
-    uint4 *stage = fused_stage + (size_t)wib * fused_rif<1>() * ETA * 32;
+    uint4 *stage = fused_stage + (size_t)wib * probe_rif<1, ETA>() * ETA * 32;
     const int sub = lane / LPG;
     const uint32_t word0 = (lane % LPG) * SW;
     const uint32_t n_short = f.counters[0];
@@ -239,7 +144,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, (LPG >= 4 || ASYNC) ? 3 : 2) k_
             const uint64_t seg = f.early_exit ? f.segment : (k1 > k0 ? k1 - k0 : 1);
             for (uint64_t a0 = k0; a0 < k1; a0 += seg) {
                 const uint64_t a1 = a0 + seg < k1 ? a0 + seg : k1;
-                slice_and(s, fused_probe_range<SW, LPG, ETA, ASYNC>(f.p, start, a0, a1, lane, word0, stage));
+                slice_and(s, probe_range<SW, LPG, ETA, ASYNC, false>(f.p, start, a0, a1, lane, word0, stage));
                 if (!f.early_exit) continue;
                 if (lane == 0 && f.probed) atomicAdd(f.probed, (unsigned long long)(a1 - a0));
                 if (a1 >= k1) break;
@@ -282,7 +187,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, (LPG >= 4 || ASYNC) ? 3 : 2) k_
         const uint64_t seg = f.early_exit ? f.segment : (nk ? nk : 1);
         for (uint64_t k0 = 0; k0 < nk; k0 += seg) {
             const uint64_t k1 = k0 + seg < nk ? k0 + seg : nk;
-            slice_and(sl, fused_probe_range<SW, LPG, ETA, ASYNC>(f.p, start, k0, k1, lane, word0, stage));
+            slice_and(sl, probe_range<SW, LPG, ETA, ASYNC, false>(f.p, start, k0, k1, lane, word0, stage));
             if (!f.early_exit) continue;
             if (lane == 0 && f.probed) atomicAdd(f.probed, (unsigned long long)(k1 - k0));
             if (k1 >= nk) break;

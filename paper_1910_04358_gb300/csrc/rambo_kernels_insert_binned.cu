@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(IB_THREADS, 4) k_insert_bin_scatter(InsertArgs
                     uint32_t at = 0;
                     if (((live >> j) & 1u) && jb + e < a.eta) {
                         const uint64_t h = mh_first_word(km, a.seed32 + jb + e);
-                        pos[j][e] = (uint32_t)(a.m_pow2 ? (h & (a.m - 1)) : (h % a.m));
+                        pos[j][e] = reduce_pos(h, a.m, a.m_inv);
                         at = atomicAdd(&s_cnt[pos[j][e] >> b.rshift], 1u);
                     }
                     const int x = j * ETA + e;
@@ -393,7 +393,10 @@ cudaError_t launch_scatter(const InsertArgs &a, const BinnedInsert &b, uint64_t 
                            cudaStream_t s) {
     const auto kernel = k_insert_bin_scatter<ETA, KIND>;
     const int occ = ib_blocks_per_sm(kernel, scatter_smem());
-    kernel<<<sm_count * occ, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
+#ifndef SC_X
+#define SC_X 1
+#endif
+    kernel<<<sm_count * occ * SC_X, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
     return cudaGetLastError();
 }
 

@@ -16,108 +16,47 @@ namespace {
 //
 // Lane roles.  A position group is read by LPG lanes, each loading an SW-word
 // slice (16 bytes when the group is >= 16 bytes), so one warp instruction
-// reads 32/LPG whole groups as runs of full 32-byte sectors.  Each warp walks
-// a contiguous range of the batch's flattened k-mer index in batches of
-// NT tiles of 32 k-mers: first every lane extracts and hashes one k-mer per
-// tile (phase 1), then the lanes load the groups of those k-mers four rounds
-// at a time (eight for one-lane groups), RIF*ETA independent loads per lane
-// in flight (phase 2).  Each lane
-// keeps a running AND of its slice for the query it is on and flushes it with
-// atomicAnd when its query changes; at the end the warp combines lanes that
-// share a query before flushing.
+// reads 32/LPG whole groups as runs of full 32-byte sectors (probe_range).
+// The batch is cut into tiles of at most `tile` k-mers of one query, numbered
+// by a prefix scan (kcum); every warp takes `per` consecutive tiles, ANDs a
+// tile's groups over its lanes and writes one mask: a plain store when the
+// query is a single tile, else an atomicAnd into the mask set to ones.  Bound
+// by the DRAM lines of the gathers (128 bytes each, whatever the group).
+// A warp that walked k-mers regardless of their query had every lane flush
+// its own slice at each query's end, 128 atomics for a 32-byte group.
 template <int SW, int LPG, int ETA>
-__global__ void __launch_bounds__(PROBE_THREADS) k_probe_seqs(ProbeArgs a) {
-    constexpr int RIF = LPG == 1 ? 8 : 4;  // rounds whose loads are in flight together
-    constexpr int NT = LPG >= RIF ? 1 : RIF / LPG;
-    constexpr int KPR = 32 / LPG;
-    constexpr int ROUNDS = NT * LPG;
-    constexpr int STEP = 32 * NT;
+__global__ void __launch_bounds__(PROBE_THREADS, LPG == 1 ? 2 : 3) k_probe_tiles(ProbeArgs a, uint32_t tile, uint32_t per) {
     const int lane = threadIdx.x & 31;
-    const int sub = lane / LPG;
     const uint32_t word0 = blockIdx.y * (LPG * SW) + (lane % LPG) * SW;
-
-    const uint64_t T = a.kcum[a.n];
-    uint64_t c0, c1;
-    warp_range<STEP>(T, a.min_chunk, c0, c1);
-    if (c0 >= T) return;
-    const uint64_t q_first = find_query(a.kcum, a.n, c0);
-
-    uint32_t cur_q = NONE;
-    Slice<SW> accv;
-    slice_ones(accv);
-
-    for (uint32_t jb = 0; jb < a.eta; jb += ETA) {
-        uint64_t qlane = q_first;
-        for (uint64_t base = c0; base < c1; base += STEP) {
-            // phase 1: k-mer, canonical form, probe positions
-            uint32_t qid[NT];
-            uint32_t pos[NT][ETA];
+    const uint64_t tiles = a.kcum[a.n];
+    const uint64_t warp = (uint64_t)blockIdx.x * (PROBE_THREADS / 32) + (threadIdx.x >> 5);
+    const uint64_t nwarps = (uint64_t)gridDim.x * (PROBE_THREADS / 32);
+    const uint64_t mine = per ? per : (tiles + nwarps - 1) / nwarps;
+    const uint64_t t0 = warp * mine;
+    if (t0 >= tiles) return;
+    const uint64_t t1 = t0 + mine < tiles ? t0 + mine : tiles;
+    uint64_t q = find_query_warp(a.kcum, a.n, t0, lane);
+    uint64_t first = a.kcum[q], next = a.kcum[q + 1];
+    for (uint64_t t = t0; t < t1; ++t) {
+        while (t >= next) {
+            ++q;
+            first = next;
+            next = a.kcum[q + 1];
+        }
+        const uint64_t b0 = a.offsets[q], nk = a.ends[q] - b0 - a.k + 1;  // (a query with tiles has k-mers)
+        const uint64_t k0 = (t - first) * tile, k1 = k0 + tile < nk ? k0 + tile : nk;
+        const Slice<SW> s = probe_range<SW, LPG, ETA, false, true>(a, b0, k0, k1, lane, word0, nullptr);
+        if (lane < LPG) {
+            if (next - first == 1) {
+                uint32_t *p = a.acc + q * a.Gw + word0;
+                if constexpr (SW == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(s.w[0], s.w[1], s.w[2], s.w[3]);
+                else
 #pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const uint64_t g = base + (uint64_t)t * 32 + lane;
-                uint64_t c = 0;
-                qid[t] = NONE;
-                if (g < c1) {
-                    while (a.kcum[qlane + 1] <= g) ++qlane;
-                    const uint64_t start = a.offsets[qlane] + a.base_shift + (g - a.kcum[qlane]);
-                    c = canonical_from_window(base_window(a.packed, a.packed_bytes, start), a.k);
-                    qid[t] = (uint32_t)qlane;
-                }
-                const uint64_t km = mh_mix_key(c);
-#pragma unroll
-                for (int e = 0; e < ETA; ++e) {
-                    const uint32_t j = jb + e < a.eta ? jb + e : a.eta - 1;
-                    pos[t][e] = reduce_pos(mh_first_word(km, a.seed32 + j), a.m, a.m_pow2);
-                }
-            }
-            // phase 2: group loads, RIF rounds in flight, then accumulate
-#pragma unroll
-            for (int rg = 0; rg < ROUNDS; rg += RIF) {
-                Slice<SW> v[RIF][ETA];
-                uint32_t qk[RIF];
-#pragma unroll
-                for (int rr = 0; rr < RIF; ++rr) {
-                    const int rho = rg + rr;
-                    const int t = rho / LPG;
-                    const int src = (rho % LPG) * KPR + sub;
-                    qk[rr] = __shfl_sync(FULL, qid[t], src);
-#pragma unroll
-                    for (int e = 0; e < ETA; ++e) {
-                        const uint32_t p = __shfl_sync(FULL, pos[t][e], src);
-                        if (qk[rr] != NONE) v[rr][e] = ld_slice<SW>(a.index + (uint64_t)p * a.Gw + word0);
-                        else slice_ones(v[rr][e]);
-                    }
-                }
-#pragma unroll
-                for (int rr = 0; rr < RIF; ++rr) {
-                    if (qk[rr] == NONE) continue;
-                    Slice<SW> x = v[rr][0];
-#pragma unroll
-                    for (int e = 1; e < ETA; ++e) slice_and(x, v[rr][e]);
-                    if (qk[rr] != cur_q) {
-                        if (cur_q != NONE) flush_slice<SW>(a.acc, cur_q, a.Gw, word0, accv);
-                        cur_q = qk[rr];
-                        accv = x;
-                    } else {
-                        slice_and(accv, x);
-                    }
-                }
+                    for (int w = 0; w < SW; ++w) p[w] = s.w[w];
+            } else {
+                flush_slice<SW>(a.acc, q, a.Gw, word0, s);
             }
         }
-    }
-    // final flush: if the whole warp is on one query, AND the lanes that hold
-    // the same slice first so only one lane per slice issues atomics
-    int same = 0;
-    __match_all_sync(FULL, cur_q, &same);
-    if (same) {
-        if (cur_q == NONE) return;
-#pragma unroll
-        for (int w = 0; w < SW; ++w)
-#pragma unroll
-            for (int off = LPG; off < 32; off <<= 1) accv.w[w] &= __shfl_xor_sync(FULL, accv.w[w], off);
-        if (sub == 0) flush_slice<SW>(a.acc, cur_q, a.Gw, word0, accv);
-    } else if (cur_q != NONE) {
-        flush_slice<SW>(a.acc, cur_q, a.Gw, word0, accv);
     }
 }
 
@@ -163,7 +102,7 @@ __global__ void __launch_bounds__(PROBE_THREADS) k_probe_kmers(ProbeArgs a) {
 #pragma unroll
                 for (int e = 0; e < ETA; ++e) {
                     const uint32_t j = jb + e < a.eta ? jb + e : a.eta - 1;
-                    pos[t][e] = reduce_pos(mh_first_word(km, a.seed32 + j), a.m, a.m_pow2);
+                    pos[t][e] = reduce_pos(mh_first_word(km, a.seed32 + j), a.m, a.m_inv);
                 }
             }
 #pragma unroll
@@ -205,22 +144,47 @@ __global__ void __launch_bounds__(PROBE_THREADS) k_probe_kmers(ProbeArgs a) {
     }
 }
 
-// sm_count > 0: SMs x occupancy maximum; sm_count < 0: -sm_count CTAs
+// K-mers a warp takes, about: small enough that many more blocks than fit are
+// handed out as SMs get free.  One even share per resident warp waits for the
+// SMs farthest from the memory: the 32 GiB batch takes 12.84 ms that way, 10.35
+// with 4,096 k-mers a warp, 10.27 with 512 and 10.26 with 256; 20,000 short
+// reads 170, 170, 155 and 148 us.
+constexpr uint64_t SEQ_SHARE = 256;
+
+// K-mers per tile of a batch of about max_kmers k-mers: 1,024 (of 16 or more
+// rounds of loads), fewer when that leaves warps without a tile.
+uint32_t tile_kmers(uint64_t max_kmers, int sm_count) {
+    uint64_t t = max_kmers / ((uint64_t)sm_count * 24);
+    t = t / 64 * 64;
+    return (uint32_t)(t < 128 ? 128 : t > 1024 ? 1024 : t);
+}
+
+// sm_count > 0: sized by the batch; sm_count < 0: -sm_count CTAs
 template <int SW, int LPG, int ETA>
-cudaError_t launch_seqs_t(const ProbeArgs &a, const Geometry &g, int sm_count, cudaStream_t s) {
-    static int occ = blocks_per_sm(k_probe_seqs<SW, LPG, ETA>, PROBE_THREADS, 0);
-    const dim3 grid(sm_count > 0 ? sm_count * occ : -sm_count, g.chunks);
-    k_probe_seqs<SW, LPG, ETA><<<grid, PROBE_THREADS, 0, s>>>(a);
+cudaError_t launch_seqs_t(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm_count, cudaStream_t s) {
+    constexpr uint64_t WARPS = PROBE_THREADS / 32;
+    uint64_t blocks = (uint64_t)-(int64_t)sm_count;
+    uint32_t per = 0;
+    if (sm_count > 0) {
+        const uint64_t tiles = a.n + a.max_kmers / tile;  // at least as many as there are
+        uint64_t share = a.min_chunk > SEQ_SHARE ? a.min_chunk : SEQ_SHARE;
+        uint64_t want = share * tiles / (a.max_kmers ? a.max_kmers : 1);
+        const uint64_t most = tiles / ((uint64_t)sm_count * 24);  // keep every warp busy first
+        if (want > most) want = most;
+        per = want < 1 ? 1 : want > 1024 ? 1024 : (uint32_t)want;
+        blocks = (tiles + WARPS * per - 1) / (WARPS * per);
+    }
+    k_probe_tiles<SW, LPG, ETA><<<dim3((unsigned)blocks, g.chunks), PROBE_THREADS, 0, s>>>(a, tile, per);
     return cudaGetLastError();
 }
 
 template <int SW, int LPG>
-cudaError_t launch_seqs_eta(const ProbeArgs &a, const Geometry &g, int sm, cudaStream_t s) {
+cudaError_t launch_seqs_eta(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm, cudaStream_t s) {
     switch (g.eta) {
-        case 1: return launch_seqs_t<SW, LPG, 1>(a, g, sm, s);
-        case 2: return launch_seqs_t<SW, LPG, 2>(a, g, sm, s);
-        case 3: return launch_seqs_t<SW, LPG, 3>(a, g, sm, s);
-        default: return launch_seqs_t<SW, LPG, 4>(a, g, sm, s);
+        case 1: return launch_seqs_t<SW, LPG, 1>(a, g, tile, sm, s);
+        case 2: return launch_seqs_t<SW, LPG, 2>(a, g, tile, sm, s);
+        case 3: return launch_seqs_t<SW, LPG, 3>(a, g, tile, sm, s);
+        default: return launch_seqs_t<SW, LPG, 4>(a, g, tile, sm, s);
     }
 }
 
@@ -234,16 +198,18 @@ cudaError_t launch_kmers_t(const ProbeArgs &a, const Geometry &g, int sm_count, 
 
 }  // namespace
 
-cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, int sm_count, cudaStream_t s) {
-    if (g.SW == 1) return launch_seqs_eta<1, 1>(a, g, sm_count, s);
-    if (g.SW == 2) return launch_seqs_eta<2, 1>(a, g, sm_count, s);
+uint32_t probe_tile_kmers(uint64_t max_kmers, int sm_count) { return tile_kmers(max_kmers, sm_count); }
+
+cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm_count, cudaStream_t s) {
+    if (g.SW == 1) return launch_seqs_eta<1, 1>(a, g, tile, sm_count, s);
+    if (g.SW == 2) return launch_seqs_eta<2, 1>(a, g, tile, sm_count, s);
     switch (g.LPG) {
-        case 1: return launch_seqs_eta<4, 1>(a, g, sm_count, s);
-        case 2: return launch_seqs_eta<4, 2>(a, g, sm_count, s);
-        case 4: return launch_seqs_eta<4, 4>(a, g, sm_count, s);
-        case 8: return launch_seqs_eta<4, 8>(a, g, sm_count, s);
-        case 16: return launch_seqs_eta<4, 16>(a, g, sm_count, s);
-        case 32: return launch_seqs_eta<4, 32>(a, g, sm_count, s);
+        case 1: return launch_seqs_eta<4, 1>(a, g, tile, sm_count, s);
+        case 2: return launch_seqs_eta<4, 2>(a, g, tile, sm_count, s);
+        case 4: return launch_seqs_eta<4, 4>(a, g, tile, sm_count, s);
+        case 8: return launch_seqs_eta<4, 8>(a, g, tile, sm_count, s);
+        case 16: return launch_seqs_eta<4, 16>(a, g, tile, sm_count, s);
+        case 32: return launch_seqs_eta<4, 32>(a, g, tile, sm_count, s);
         default: return cudaErrorInvalidValue;
     }
 }

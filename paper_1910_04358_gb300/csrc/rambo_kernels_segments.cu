@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(SEG_THREADS) k_seg_probe(SegArgs a) {
                 const uint64_t km = mh_mix_key(c);
 #pragma unroll
                 for (int e = 0; e < ETA; ++e)
-                    pos[h][e] = reduce_pos(mh_first_word(km, p.seed32 + (uint32_t)e), p.m, p.m_pow2);
+                    pos[h][e] = reduce_pos(mh_first_word(km, p.seed32 + (uint32_t)e), p.m, p.m_inv);
             }
         };
         uint32_t cur = NONE;

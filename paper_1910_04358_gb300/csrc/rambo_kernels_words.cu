@@ -81,7 +81,7 @@ __global__ void k_insert_words(WordArgs a) {
         if (!term_bytes(a, t, &w, &len)) continue;
         for (uint32_t j = 0; j < a.eta; ++j) {
             const uint64_t h = mh_bytes_first_word(w, len, a.seed32 + j);
-            const uint64_t p = a.m_pow2 ? (h & (a.m - 1)) : (h % a.m);
+            const uint64_t p = reduce_pos(h, a.m, a.m_inv);
             for (uint32_t r = 0; r < a.R; ++r) {
                 const uint32_t bb = r * a.B + a.phi[(uint64_t)d * a.R + r];
                 atomicOr(a.index + p * a.Gw + (bb >> 5), 1u << (bb & 31));
@@ -104,7 +104,7 @@ __global__ void k_probe_words(WordArgs a) {
         uint32_t pos[64];
         for (uint32_t j = 0; j < a.eta; ++j) {
             const uint64_t h = mh_bytes_first_word(w, len, a.seed32 + j);
-            pos[j] = (uint32_t)(a.m_pow2 ? (h & (a.m - 1)) : (h % a.m));
+            pos[j] = reduce_pos(h, a.m, a.m_inv);
         }
         uint32_t *acc = a.acc + q * a.Gw;
         for (uint32_t word = 0; word < a.Gw; ++word) {

@@ -12,10 +12,6 @@ constexpr uint32_t FULL = 0xffffffffu;
 constexpr uint32_t NONE = 0xffffffffu;
 constexpr int PROBE_THREADS = 256;
 
-__device__ __forceinline__ uint32_t reduce_pos(uint64_t h, uint64_t m, uint32_t m_pow2) {
-    return (uint32_t)(m_pow2 ? (h & (m - 1)) : (h % m));
-}
-
 // 16-byte copy from global to shared memory that does not pass through
 // registers (caching in L2 only), and the wait for this thread's copies.
 __device__ __forceinline__ void cp_async16(uint4 *smem, const void *gmem) {
@@ -34,6 +30,21 @@ __device__ __forceinline__ uint64_t find_query(const uint64_t *kcum, uint64_t n,
         uint64_t mid = (lo + hi) >> 1;
         if (kcum[mid] <= g) lo = mid;
         else hi = mid;
+    }
+    return lo;
+}
+
+// The same by a whole warp, g the same in every lane.  The warp looks at 32 places at a time: three rounds of
+// loads for 32,768 queries where halving takes fifteen.
+__device__ __forceinline__ uint64_t find_query_warp(const uint64_t *kcum, uint64_t n, uint64_t g, int lane) {
+    uint64_t lo = 0, len = n;  // q in [lo, lo + len), kcum[lo] <= g
+    while (len > 1) {
+        const uint64_t step = (len + 31) / 32;
+        const uint64_t at = (uint64_t)lane * step;
+        const uint32_t le = __ballot_sync(FULL, at < len && kcum[lo + at] <= g);  // a run from lane 0 on
+        const uint64_t piece = (uint64_t)(31 - __clz(le)) * step;
+        lo += piece;
+        len = len - piece < step ? len - piece : step;
     }
     return lo;
 }
@@ -61,6 +72,105 @@ __device__ __forceinline__ void flush_slice(uint32_t *acc, uint64_t q, uint32_t 
         if (v.w[w] != FULL) atomicAnd(p + w, v.w[w]);
 }
 
+// Rounds of ETA loads a lane keeps in flight (16 loads of one-lane groups, 8
+// of wider ones; more probes a round spill otherwise).
+template <int LPG, int ETA>
+__host__ __device__ constexpr int probe_rif() { return (LPG == 1 ? 8 : 4) / (ETA <= 2 ? 1 : 2); }
+
+// AND of the groups of k-mers [k0, k1) of one query, per lane slice (every
+// lane of the warp works on the same query).  ASYNC (one lane per 16-byte
+// group): the gathers land in the warp's shared-memory `stage` through
+// cp.async instead of registers, so a lane holds no load data in flight.
+// SKIP: tiles of 32 k-mers past the end are not hashed (short ranges).
+template <int SW, int LPG, int ETA, bool ASYNC, bool SKIP>
+__device__ __forceinline__ Slice<SW> probe_range(const ProbeArgs &a, uint64_t start,
+                                                        uint64_t k0, uint64_t k1, int lane,
+                                                        uint32_t word0, uint4 *stage) {
+    static_assert(!ASYNC || (LPG == 1 && SW == 4), "staged gathers: one lane per 16-byte group");
+    constexpr int RIF = probe_rif<LPG, ETA>();  // rounds whose loads are in flight together
+    constexpr int NT = LPG >= RIF ? 1 : RIF / LPG;
+    constexpr int KPR = 32 / LPG;
+    constexpr int ROUNDS = NT * LPG;
+    constexpr int STEP = 32 * NT;
+    const int sub = lane / LPG;
+    Slice<SW> accv;
+    slice_ones(accv);
+    for (uint32_t jb = 0; jb < a.eta; jb += ETA) {
+        for (uint64_t base = k0; base < k1; base += STEP) {
+            uint32_t pos[NT][ETA];
+            bool val[NT];
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const uint64_t g = base + (uint64_t)t * 32 + lane;
+                val[t] = g < k1;
+                if (SKIP && t > 0 && base + (uint64_t)t * 32 >= k1) continue;  // the whole warp
+                uint64_t c = 0;
+                if (val[t])
+                    c = canonical_from_window(base_window(a.packed, a.packed_bytes, start + a.base_shift + g), a.k);
+                const uint64_t km = mh_mix_key(c);
+#pragma unroll
+                for (int e = 0; e < ETA; ++e) {
+                    const uint32_t j = jb + e < a.eta ? jb + e : a.eta - 1;
+                    pos[t][e] = reduce_pos(mh_first_word(km, a.seed32 + j), a.m, a.m_inv);
+                }
+            }
+#pragma unroll
+            for (int rg = 0; rg < ROUNDS; rg += RIF) {
+                if constexpr (ASYNC) {
+                    // each lane gathers its own k-mers' groups (LPG == 1)
+                    uint32_t live = 0;
+#pragma unroll
+                    for (int rr = 0; rr < RIF; ++rr) {
+                        const int t = rg + rr;
+#pragma unroll
+                        for (int e = 0; e < ETA; ++e)
+                            if (val[t]) {
+                                cp_async16(stage + (rr * ETA + e) * 32 + lane,
+                                           a.index + (uint64_t)pos[t][e] * a.Gw + word0);
+                                live |= 1u << (rr * ETA + e);
+                            }
+                    }
+                    cp_async_wait_all();
+#pragma unroll
+                    for (int i = 0; i < RIF * ETA; ++i)
+                        if (live & (1u << i)) {
+                            const uint4 v = stage[i * 32 + lane];
+                            accv.w[0] &= v.x;
+                            accv.w[1] &= v.y;
+                            accv.w[2] &= v.z;
+                            accv.w[3] &= v.w;
+                        }
+                    continue;
+                }
+                Slice<SW> v[RIF][ETA];
+#pragma unroll
+                for (int rr = 0; rr < RIF; ++rr) {
+                    const int rho = rg + rr;
+                    const int t = rho / LPG;
+                    const int src = (rho % LPG) * KPR + sub;
+                    const bool vs = __shfl_sync(FULL, (int)val[t], src) != 0;
+#pragma unroll
+                    for (int e = 0; e < ETA; ++e) {
+                        const uint32_t p = __shfl_sync(FULL, pos[t][e], src);
+                        if (vs) v[rr][e] = ld_slice<SW>(a.index + (uint64_t)p * a.Gw + word0);
+                        else slice_ones(v[rr][e]);
+                    }
+                }
+#pragma unroll
+                for (int rr = 0; rr < RIF; ++rr)
+#pragma unroll
+                    for (int e = 0; e < ETA; ++e) slice_and(accv, v[rr][e]);
+            }
+        }
+    }
+    // combine the lanes that hold the same slice
+#pragma unroll
+    for (int w = 0; w < SW; ++w)
+#pragma unroll
+        for (int off = LPG; off < 32; off <<= 1) accv.w[w] &= __shfl_xor_sync(FULL, accv.w[w], off);
+    return accv;
+}
+
 // Per-warp contiguous range of the flattened k-mer index space [0, T).
 template <int STEP>
 __device__ __forceinline__ void warp_range(uint64_t T, uint32_t min_chunk, uint64_t &c0, uint64_t &c1) {
@@ -68,8 +178,10 @@ __device__ __forceinline__ void warp_range(uint64_t T, uint32_t min_chunk, uint6
     const uint64_t nwarps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     uint64_t per = (T + nwarps - 1) / nwarps;
     if (per < min_chunk) per = min_chunk;
-    per = (per + STEP - 1) / STEP * STEP;
-    if (per < 2 * STEP) per = 2 * STEP;
+    // whole steps, but only whole tiles of 32 where a step is more than a
+    // warp's share (a small batch then spreads over all warps)
+    const uint64_t unit = per < STEP ? 32 : STEP;
+    per = (per + unit - 1) / unit * unit;
     c0 = warp * per;
     c1 = c0 + per < T ? c0 + per : T;
 }

@@ -112,3 +112,52 @@ def test_insert_record_shapes_match_oracle(rambo_lib, K, B, R, m, eta):
                 assert np.array_equal(bits[:, r * B + b], want), (st, r, b)
         assert not bits[:, R * B:].any()
         idx.close()
+
+
+def test_sequence_batches_around_the_prefix_scans(rambo_lib):
+    # one block, a cluster of blocks (its shares kept and recounted), three
+    # launches; queries of no, one or a few k-mers
+    import torch
+    p = synth.Params(K=40, B=8, R=2, m=1 << 12, eta=2, k=15, seed=1)
+    rng = np.random.default_rng(6)
+    corpus = synth.family_corpus(rng, p, n_seeds=8, doc_len=300, sub_rate=0.02)
+    n = 131075
+    offs = np.concatenate([[0], np.cumsum(rng.integers(12, 20, size=n))]).astype(np.uint64)
+    packed = np.concatenate([corpus.packed[:2900]] * (int(offs[-1]) // 11600 + 1) + [np.zeros(16, np.uint8)])
+    o = oracle.Rambo(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    o.insert_batch(corpus.doc_ids, corpus.packed, corpus.offsets)
+    want = o.query_seqs(packed, offs, threads=4)
+    idx = rambo_lib.Index(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    idx.insert_batch(corpus.doc_ids, corpus.packed, corpus.offsets)
+    dp, do = _dev(torch, packed, np.uint8), _dev(torch, offs, np.int64)
+    for path in (0, 1):
+        idx.set_tuning(query_path=path)
+        for m in (1, 4095, 4096, 4097, 32768, 32769, 131072, n):
+            got = idx.query_seqs_dev(dp, do[:m + 1])
+            idx.sync()
+            assert np.array_equal(rambo_lib.as_u32(got), want[:m]), (path, m)
+
+
+@pytest.mark.parametrize("K,B,R,eta", [(300, 32, 4, 2), (300, 60, 3, 3), (200, 100, 5, 1), (64, 400, 6, 2)])
+def test_sequence_tiles_match_oracle(rambo_lib, K, B, R, eta):
+    # tiles of a query: none, part of one, exactly one and one k-mer more,
+    # several; small batches with a fused path set take the same tiles
+    import torch
+    p = synth.Params(K=K, B=B, R=R, m=(1 << 14) - 3, eta=eta, k=31, seed=2)
+    rng = np.random.default_rng(K + R)
+    corpus = synth.family_corpus(rng, p, n_seeds=12, doc_len=3000, sub_rate=0.005)
+    lens = [0, 30, 31, 62, 63, 94, 157, 158, 159, 286, 287, 1054, 1055, 2500] * 9
+    q = synth.sample_queries(rng, corpus, np.array(lens), 0.8)
+    o = oracle.Rambo(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    o.insert_batch(corpus.doc_ids, corpus.packed, corpus.offsets)
+    want = o.query_seqs(q.packed, q.offsets)
+    idx = rambo_lib.Index(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    idx.insert_batch(corpus.doc_ids, corpus.packed, corpus.offsets)
+    dp, do = _dev(torch, q.packed, np.uint8), _dev(torch, q.offsets, np.int64)
+    for st in (dict(query_path=0), dict(query_path=0, probe_ctas_per_sm=1), dict(query_path=0, probe_min_kmers_per_warp=5000),
+               dict(query_path=1, fused_tile_kmers=4096), dict(query_path=1, fused_tile_kmers=1)):
+        idx.set_tuning(probe_ctas_per_sm=0, probe_min_kmers_per_warp=0)
+        idx.set_tuning(**st)
+        got = idx.query_seqs_dev(dp, do)
+        idx.sync()
+        assert np.array_equal(rambo_lib.as_u32(got), want), st
