@@ -388,15 +388,16 @@ int ib_blocks_per_sm(KernelT kernel, size_t smem) {
     return n;
 }
 
+// Blocks per resident block, as in the direct insertion (medium build: 21.8 ms
+// with 1, 21.1 with 4, 20.7 with 16, 20.8 with 32).
+constexpr int SCATTER_WAVES = 16;
+
 template <int ETA, int KIND>
 cudaError_t launch_scatter(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1, int sm_count,
                            cudaStream_t s) {
     const auto kernel = k_insert_bin_scatter<ETA, KIND>;
     const int occ = ib_blocks_per_sm(kernel, scatter_smem());
-#ifndef SC_X
-#define SC_X 1
-#endif
-    kernel<<<sm_count * occ * SC_X, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
+kernel<<<sm_count * occ * SCATTER_WAVES, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
     return cudaGetLastError();
 }
 
