@@ -9,6 +9,7 @@ module raises.
 from __future__ import annotations
 
 import ctypes as C
+import itertools
 import threading
 
 import numpy as np
@@ -405,43 +406,54 @@ class Index:
 
     # ------------------------------------------------ documents of words
     @staticmethod
-    def _word_batch(items):
-        """CSR buffers for a list of items, each a list of byte strings."""
+    def _word_batch(items, stream):
+        """CSR buffers for a list of items, each a list of byte strings, copied to
+        the device on `stream` as one page-locked buffer (three pageable copies
+        each wait for the device).  Returns (the device buffer, addresses of the
+        bytes, the term offsets and the item offsets, bytes)."""
         import torch
-        words = [w for it in items for w in it]
-        buf = np.frombuffer(b"".join(words) + b"\0" * 8, dtype=np.uint8).copy()
-        term_offs = np.zeros(len(words) + 1, dtype=np.int64)
-        if words:
-            term_offs[1:] = np.cumsum([len(w) for w in words])
-        item_terms = np.zeros(len(items) + 1, dtype=np.int64)
-        item_terms[1:] = np.cumsum([len(it) for it in items])
-        dev = lambda a: torch.from_numpy(a).cuda()
-        return dev(buf), int(term_offs[-1]), dev(term_offs), dev(item_terms)
+        words = list(itertools.chain.from_iterable(items))
+        text = b"".join(words)
+        t0 = (len(text) + 15) // 8 * 8          # at least 8 zero bytes behind the last word
+        i0 = t0 + 8 * (len(words) + 1)
+        host = torch.empty(i0 + 8 * (len(items) + 1), dtype=torch.uint8, pin_memory=True)
+        h = host.numpy()
+        h[:len(text)] = np.frombuffer(text, dtype=np.uint8)
+        h[len(text):t0] = 0
+        for at, of in ((t0, words), (i0, items)):
+            offs = h[at:at + 8 * (len(of) + 1)].view(np.int64)
+            offs[0] = 0
+            np.cumsum(np.fromiter(map(len, of), dtype=np.int64, count=len(of)), out=offs[1:])
+        with torch.cuda.stream(stream):
+            buf = host.to("cuda", non_blocking=True)
+        p = buf.data_ptr()
+        return buf, p, p + t0, p + i0, len(text)
 
     def insert_words(self, doc_ids, docs, stream=None):
         """docs[i]: list of byte strings (the words of document doc_ids[i])."""
         import torch
-        buf, nbytes, toffs, iterms = self._word_batch(docs)
         ids = torch.from_numpy(np.ascontiguousarray(doc_ids, dtype=np.uint32).view(np.int32)).cuda()
-        _check(load().rambo_insert_words_dev(self._h, len(docs), _t_ptr(ids), _t_ptr(buf), nbytes,
-                                             _t_ptr(toffs), _t_ptr(iterms), _stream_handle(stream)),
-               "rambo_insert_words_dev")
+        buf, text, toffs, iterms, nbytes = self._word_batch(docs, stream)
+        _check(load().rambo_insert_words_dev(self._h, len(docs), _t_ptr(ids), text, nbytes, toffs, iterms,
+                                             _stream_handle(stream)), "rambo_insert_words_dev")
         self.sync(stream)
 
     def query_words(self, queries, stream=None) -> np.ndarray:
         """queries[i]: list of byte strings; returns (n, W) uint32 masks."""
         import torch
-        buf, nbytes, toffs, iterms = self._word_batch(queries)
+        buf, text, toffs, iterms, nbytes = self._word_batch(queries, stream)
         n = len(queries)
-        out = torch.empty((n, self.W), dtype=torch.int32, device="cuda")
         s = _stream_handle(stream)
-        need = int(load().rambo_query_words_workspace(self._h, n))
-        wp, wn = self._workspace(("words", s), need)
-        _check(load().rambo_query_words_dev(self._h, n, _t_ptr(buf), nbytes, _t_ptr(toffs),
-                                            _t_ptr(iterms), _t_ptr(out), wp, wn, s),
-               "rambo_query_words_dev")
+        with torch.cuda.stream(stream):
+            out = torch.empty((n, self.W), dtype=torch.int32, device="cuda")
+            need = int(load().rambo_query_words_workspace(self._h, n))
+            wp, wn = self._workspace(("words", s), need)
+            _check(load().rambo_query_words_dev(self._h, n, text, nbytes, toffs, iterms, _t_ptr(out), wp, wn, s),
+                   "rambo_query_words_dev")
+            host = torch.empty((n, self.W), dtype=torch.int32, pin_memory=True)
+            host.copy_(out, non_blocking=True)
         self.sync(stream)
-        return as_u32(out)
+        return host.numpy().view(np.uint32)
 
     # ------------------------------------------------------------ folding
     def fold(self):
