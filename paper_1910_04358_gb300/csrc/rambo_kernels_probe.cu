@@ -31,7 +31,10 @@ __global__ void __launch_bounds__(PROBE_THREADS, LPG == 1 ? 2 : 3) k_probe_tiles
     const uint64_t tiles = a.kcum[a.n];
     const uint64_t warp = (uint64_t)blockIdx.x * (PROBE_THREADS / 32) + (threadIdx.x >> 5);
     const uint64_t nwarps = (uint64_t)gridDim.x * (PROBE_THREADS / 32);
-    const uint64_t mine = per ? per : (tiles + nwarps - 1) / nwarps;
+    // (`per` comes from the bases the batch is known to span; items that overlap
+    // have more tiles, which the warps then share evenly)
+    const uint64_t even = (tiles + nwarps - 1) / nwarps;
+    const uint64_t mine = per > even ? per : even;
     const uint64_t t0 = warp * mine;
     if (t0 >= tiles) return;
     const uint64_t t1 = t0 + mine < tiles ? t0 + mine : tiles;
@@ -166,7 +169,7 @@ cudaError_t launch_seqs_t(const ProbeArgs &a, const Geometry &g, uint32_t tile, 
     uint64_t blocks = (uint64_t)-(int64_t)sm_count;
     uint32_t per = 0;
     if (sm_count > 0) {
-        const uint64_t tiles = a.n + a.max_kmers / tile;  // at least as many as there are
+        const uint64_t tiles = a.n + a.max_kmers / tile;  // at least as many as items that do not overlap have
         uint64_t share = a.min_chunk > SEQ_SHARE ? a.min_chunk : SEQ_SHARE;
         uint64_t want = share * tiles / (a.max_kmers ? a.max_kmers : 1);
         const uint64_t most = tiles / ((uint64_t)sm_count * 24);  // keep every warp busy first

@@ -161,3 +161,30 @@ def test_sequence_tiles_match_oracle(rambo_lib, K, B, R, eta):
         got = idx.query_seqs_dev(dp, do)
         idx.sync()
         assert np.array_equal(rambo_lib.as_u32(got), want), st
+
+
+@pytest.mark.parametrize("path", [0, 1])
+def test_overlapping_ranges_have_more_tiles_than_bases(rambo_lib, path):
+    # 2,000 ranges over the same 4,000 bases: sixteen times the tiles that the
+    # buffer's length suggests
+    import torch
+    p = synth.Params(K=60, B=16, R=3, m=1 << 14, eta=2, k=31, seed=12)
+    rng = np.random.default_rng(9)
+    corpus = synth.family_corpus(rng, p, n_seeds=4, doc_len=4000, sub_rate=0.002)
+    idx = rambo_lib.Index(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    idx.insert_batch(corpus.doc_ids, corpus.packed, corpus.offsets)
+    o = oracle.Rambo(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    o.insert_batch(corpus.doc_ids, corpus.packed, corpus.offsets)
+    # most of a document, then bases of none: ranges past it have no answer
+    packed = synth.pack_bases(np.concatenate([corpus.doc_bases(0)[:3500], synth.uniform_genome(rng, 500)]))
+    begins = rng.integers(0, 100, size=2000)
+    ends = rng.integers(3000, 4001, size=2000)
+    seqs = [synth.unpack_bases(packed, int(b), int(e - b)) for b, e in zip(begins, ends)]
+    qp, qo = synth.pack_many(seqs)
+    want = o.query_seqs(qp, qo, threads=4)
+    idx.set_tuning(query_path=path)
+    got = idx.query_ranges_dev(_dev(torch, packed, np.uint8), _dev(torch, begins.astype(np.int64), np.int64),
+                               _dev(torch, ends.astype(np.int64), np.int64))
+    idx.sync()
+    assert np.array_equal(rambo_lib.as_u32(got), want)
+    assert 0 < want.any(axis=1).sum() < 2000
