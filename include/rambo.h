@@ -399,12 +399,9 @@ typedef struct {
                                        /* many CTAs per SM (0 = as probe_ctas_per_sm;  */
                                        /* default 1), leaving room for the k-mer       */
                                        /* chunks whose copies out bound the call       */
-    uint32_t insert_mode;              /* Algorithm 1's bit setting: 0 = lanes hitting */
-                                       /* one word combine first (match + OR-reduce);  */
-                                       /* 1 = one 32-bit atomicOr per repetition; 2    */
-                                       /* (default) = as 1 with repetitions that share */
-                                       /* a 64-bit word merged into one 64-bit         */
-                                       /* atomicOr (32-bit when m * Gw is odd); 3 =    */
+    uint32_t insert_mode;              /* Algorithm 1's bit setting: 0, 1, 2 (default) =  */
+                                       /* direct: neighbouring lanes set one probe's   */
+                                       /* repetitions or 64-bit words together; 3 =    */
                                        /* binned by index region (bin_region_kib):     */
                                        /* probes are first written as 8-byte records   */
                                        /* per region, then applied region by region so */
