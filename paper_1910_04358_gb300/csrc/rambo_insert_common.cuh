@@ -21,7 +21,8 @@ constexpr uint32_t NO_DOC = 0xffffffffu;
 // 22.9 and 193).
 //   KIND 0  repetitions, 32-bit words, buckets from phi
 //   KIND 1  the 64-bit words of the group, from the documents' patterns
-//           (at most R / 2 of them, so that nearly all have a bit)
+//           (at most R / 2 of them, so that nearly all have a bit, and at
+//           most 32)
 //   KIND 2  the one 32-bit word of a 4-byte group, from its pattern
 template <int KIND>
 struct RecordSetter {

@@ -227,7 +227,7 @@ struct InsertArgs {
     const unsigned long long *pattern;  // pattern_bytes: the documents' group words, or null
     uint32_t kind;             // RecordSetter: 0 = a lane per repetition, 1 = per 64-bit word,
                                // 2 = one 32-bit word
-    uint32_t lanes;            // lanes per record
+    uint32_t lanes;            // lanes per record, 1..32
 };
 
 // Word documents (Section 5.4): term t is bytes [term_offs[t], term_offs[t+1])
@@ -284,8 +284,10 @@ cudaError_t launch_insert(const InsertArgs &a, int sm_count, cudaStream_t s);
 // where records are set word by word: 4-byte groups, and groups of at most R
 // 32-bit words, where a lane per 64-bit word needs at most half the lanes of
 // one per repetition (16-byte groups with R = 4 in L2: 207 against 201 G
-// records/s).  Wider groups give 0 and are set repetition by repetition
-// (32-byte groups with R = 5: 151 against 130; equal in DRAM).
+// records/s), and of at most 64, so that a warp's lanes hold a whole record
+// (R of 128 and more reach groups past that).  Wider groups give 0 and are set
+// repetition by repetition (32-byte groups with R = 5: 151 against 130; equal
+// in DRAM).
 uint64_t pattern_bytes(const Geometry &g);
 cudaError_t launch_patterns(const Geometry &g, unsigned long long *pattern, const uint32_t *phi, cudaStream_t s);
 // ORs the answers of one document shard (n rows of shard_words words, bit j

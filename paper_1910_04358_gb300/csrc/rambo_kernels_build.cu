@@ -466,7 +466,7 @@ cudaError_t launch_fold(const uint32_t *old_index, uint32_t old_gw, uint32_t *ne
 
 uint64_t pattern_bytes(const Geometry &g) {
     if (g.Gw == 1) return (uint64_t)g.K * 4;
-    return g.Gw <= g.R ? (uint64_t)g.K * (g.Gw / 2) * 8 : 0;
+    return g.Gw <= g.R && g.Gw <= 64 ? (uint64_t)g.K * (g.Gw / 2) * 8 : 0;
 }
 
 cudaError_t launch_patterns(const Geometry &g, unsigned long long *pattern, const uint32_t *phi, cudaStream_t s) {
@@ -476,6 +476,7 @@ cudaError_t launch_patterns(const Geometry &g, unsigned long long *pattern, cons
 }
 
 cudaError_t launch_insert(const InsertArgs &a, int sm_count, cudaStream_t s) {
+    if (a.lanes < 1 || a.lanes > 32) return cudaErrorInvalidValue;  // a turn holds at least one record
     switch (a.eta) {
         case 1: return launch_insert_t<1>(a, sm_count, s);
         case 2: return launch_insert_t<2>(a, sm_count, s);

@@ -441,6 +441,7 @@ uint32_t binned_insert_bins(uint64_t m, uint32_t group_bytes, uint32_t K, uint64
 
 cudaError_t launch_insert_binned(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1,
                                  int sm_count, cudaStream_t s) {
+    if (a.lanes < 1 || a.lanes > 32) return cudaErrorInvalidValue;  // a turn holds at least one record
     switch (a.kind) {
         case 0: return launch_binned_k<0>(a, b, f0, f1, sm_count, s);
         case 1: return launch_binned_k<1>(a, b, f0, f1, sm_count, s);

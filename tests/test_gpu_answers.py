@@ -114,6 +114,17 @@ def test_insert_record_shapes_match_oracle(rambo_lib, K, B, R, m, eta):
         idx.close()
 
 
+@pytest.mark.parametrize("K,B,R,m,eta", [
+    (60, 16, 128, 1 << 12, 2),    # 256-byte groups, the most words a warp sets at once
+    (60, 17, 128, 1 << 12, 2),    # 512-byte groups: a lane per repetition
+    (60, 20, 128, 4093, 1),
+    (50, 9, 256, 1 << 12, 3),     # 512-byte groups, eight repetitions a lane
+    (40, 10, 500, 1 << 11, 2),    # groups of two 512-byte chunks
+])
+def test_insert_records_of_many_repetitions_match_oracle(rambo_lib, K, B, R, m, eta):
+    test_insert_record_shapes_match_oracle(rambo_lib, K, B, R, m, eta)
+
+
 def test_sequence_batches_around_the_prefix_scans(rambo_lib):
     # one block, a cluster of blocks (its shares kept and recounted), three
     # launches; queries of no, one or a few k-mers

@@ -1,9 +1,11 @@
 """Host-side helpers (no GPU): answer-mask decoding and the bench's choice of
 the query path the library takes."""
+import ctypes
+
 import numpy as np
 
 import oracle
-from paper_1910_04358_gb300 import rambo
+from paper_1910_04358_gb300 import build, rambo
 
 
 def test_answer_docs_matches_oracle_mask_decoding():
@@ -136,3 +138,30 @@ def test_serving_trace_refuses_requests_beyond_the_batch_bytes():
         serve._Trace([small, big], max_bytes=4096)
     with pytest.raises(ValueError):  # ids must be 0 .. n-1
         serve._Trace([serve.Request(3, np.zeros(4, np.uint8), 16, 0.0)], max_bytes=4096)
+
+
+class _Geometry(ctypes.Structure):
+    _fields_ = [(f, ctypes.c_uint32) for f in ("K", "B", "R", "eta", "k")] + [
+        ("m", ctypes.c_uint64), ("seed", ctypes.c_uint64)] + [
+        (f, ctypes.c_uint32) for f in ("W", "gbits", "Gw", "SW", "LPG", "chunks")]
+
+
+def test_a_warp_holds_a_whole_insert_record():
+    # rgpu::make_geometry and rgpu::pattern_bytes: groups that are set word by
+    # word have at most 32 words of 64 bits, a lane each
+    lib = ctypes.CDLL(build.build())
+    geometry = lib._ZN4rgpu13make_geometryEjjjmjjm
+    geometry.restype = _Geometry
+    geometry.argtypes = [ctypes.c_uint32] * 3 + [ctypes.c_uint64] + [ctypes.c_uint32] * 2 + [ctypes.c_uint64]
+    pattern_bytes = lib._ZN4rgpu13pattern_bytesERKNS_8GeometryE
+    pattern_bytes.restype = ctypes.c_uint64
+    by_word = 0
+    for R in list(range(1, 513)) + [1000, 4096, 100_000]:
+        for B in (1, 2, 3, 4, 8, 9, 15, 16, 17, 20, 31, 32, 33, 64, 100):
+            g = geometry(10, B, R, 1 << 10, 2, 31, 0)
+            bits = pattern_bytes(ctypes.byref(g))
+            lanes = min(R, 32) if bits == 0 else max(g.Gw // 2, 1)
+            assert bits in (0, 10 * (8 * lanes if g.Gw > 1 else 4)), (R, B)
+            assert 1 <= lanes <= 32, (R, B, g.Gw)
+            by_word += bits > 0
+    assert by_word > 100
