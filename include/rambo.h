@@ -297,8 +297,8 @@ int rambo_sync(rambo_t *h, void *stream);
  * stacked, document-sharded deployment is expressed as one index (Section
  * 5.3: bucket b*tau(D) + phi_i(D) over S shards of b buckets each).  Allowed
  * only before the first insert (RAMBO_ESTATE afterwards); RAMBO_EINVAL if a
- * bucket is out of range.  Folding afterwards recomputes the default
- * partition. */
+ * bucket is out of range.  Folding afterwards folds the map with the index:
+ * bucket b+B/2 becomes b. */
 int rambo_set_partition(rambo_t *h, const uint32_t *phi);
 
 /* ---------------------------------------------------------------------- */

@@ -1386,8 +1386,9 @@ int rambo_fold(rambo_t *h) {
     if (!rc) rc = cuda_rc(cudaMalloc(&np, (uint64_t)ng.K * ng.R * 4));
     if (!rc) rc = cuda_rc(launch_fold(h->d_index, old.Gw, ni, ng.Gw, old.m, old.B, old.R, h->d_docbits,
                                       nd, old.W, h->sm_count, h->stream));
-    // the folded partition is phi_r(d) mod B/2 = hash mod B/2, since B/2 divides B
-    if (!rc) rc = cuda_rc(launch_partition(np, ng.K, ng.R, ng.B, ng.seed, h->stream));
+    // the folded partition is phi_r(d) mod B/2, of an explicit map too; of the
+    // default map it is the hash mod B/2, since B/2 divides B
+    if (!rc) rc = cuda_rc(launch_fold_partition(np, h->d_phi, ng.K, ng.R, ng.B, h->stream));
     // the documents' slots of the folded geometry
     const uint64_t slot_words = answer_slot_words(ng);
     if (!rc && slot_words) rc = cuda_rc(cudaMalloc(&ns, slot_words * 4));

@@ -256,6 +256,9 @@ cudaError_t launch_probe_words(const WordArgs &a, int sm_count, cudaStream_t s);
 // status.
 cudaError_t launch_partition(uint32_t *phi, uint32_t K, uint32_t R, uint32_t B, uint64_t seed,
                              cudaStream_t s);
+// folded[i] = phi[i] mod Bh: the documents' buckets in an index folded to Bh.
+cudaError_t launch_fold_partition(uint32_t *folded, const uint32_t *phi, uint32_t K, uint32_t R, uint32_t Bh,
+                                  cudaStream_t s);
 // Exclusive prefix (n+1 values) of the k-mer counts of items
 // [begins[i], ends[i]); with tile > 0, of the tile counts of the items with
 // more than short_max k-mers (ceil(k-mers / tile); shorter items count 0).

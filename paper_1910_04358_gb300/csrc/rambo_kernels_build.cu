@@ -27,6 +27,13 @@ __global__ void k_partition(uint32_t *phi, uint32_t K, uint32_t R, uint32_t B, u
     phi[i] = (uint32_t)(h % B);
 }
 
+// The partition of an index folded to Bh buckets: bucket b + Bh's documents
+// join bucket b, whatever map they were placed by.
+__global__ void k_fold_partition(uint32_t *folded, const uint32_t *phi, uint64_t n, uint32_t Bh) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) folded[i] = phi[i] % Bh;
+}
+
 // -------------------------------------------------------------- prefix scan
 constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_ITEMS = 16;
@@ -412,6 +419,13 @@ cudaError_t launch_partition(uint32_t *phi, uint32_t K, uint32_t R, uint32_t B, 
                              cudaStream_t s) {
     const uint64_t n = (uint64_t)K * R;
     k_partition<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(phi, K, R, B, seed);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fold_partition(uint32_t *folded, const uint32_t *phi, uint32_t K, uint32_t R, uint32_t Bh,
+                                  cudaStream_t s) {
+    const uint64_t n = (uint64_t)K * R;
+    k_fold_partition<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(folded, phi, n, Bh);
     return cudaGetLastError();
 }
 

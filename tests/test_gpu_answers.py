@@ -199,3 +199,47 @@ def test_overlapping_ranges_have_more_tiles_than_bases(rambo_lib, path):
     idx.sync()
     assert np.array_equal(rambo_lib.as_u32(got), want)
     assert 0 < want.any(axis=1).sum() < 2000
+
+
+def _all_paths_match(rambo_lib, torch, idx, o, kmers, q):
+    dk, dp, do = _dev(torch, kmers, np.int64), _dev(torch, q.packed, np.uint8), _dev(torch, q.offsets, np.int64)
+    want, want_k = o.query_seqs(q.packed, q.offsets), o.query_kmers(kmers)
+    # (early exit keeps a batch of any size on the persistent launch)
+    for st in (dict(query_path=0), dict(query_path=1, early_exit=1), dict(query_path=2, early_exit=0), dict(query_path=3)):
+        idx.set_tuning(**st)
+        got, got_k = idx.query_seqs_dev(dp, do), idx.query_kmers_dev(dk)
+        idx.sync()
+        assert np.array_equal(rambo_lib.as_u32(got), want), st
+        assert np.array_equal(rambo_lib.as_u32(got_k), want_k), st
+    return want
+
+
+@pytest.mark.parametrize("K,B,R", [(120, 16, 3), (300, 60, 4), (70, 8, 8)])
+def test_fold_of_an_explicit_partition(rambo_lib, K, B, R):
+    import torch
+    p = synth.Params(K=K, B=B, R=R, m=1 << 12, eta=2, k=21, seed=9)
+    rng = np.random.default_rng(K * B + R)
+    corpus = synth.family_corpus(rng, p, n_seeds=max(1, K // 12), doc_len=200, sub_rate=0.02)
+    q = synth.sample_queries(rng, corpus, rng.integers(15, 150, size=150), 0.8)
+    kmers = synth.sample_kmers(rng, corpus, 300, p.k, 0.8)
+    phi = rng.integers(0, B, size=(K, R)).astype(np.uint32)
+    o = oracle.Rambo(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    idx = rambo_lib.Index(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    for x in (o, idx):
+        x.set_partition(phi)
+
+    def insert(ids):
+        packed, offs = synth.pack_many([corpus.doc_bases(int(d)) for d in ids])
+        for x in (o, idx):
+            x.insert_batch(np.asarray(ids, dtype=np.uint32), packed, offs)
+
+    insert(corpus.doc_ids[::2])
+    for fold in (False, True, True):
+        if fold:
+            idx.fold()
+            o.fold()
+        assert _all_paths_match(rambo_lib, torch, idx, o, kmers, q).any()
+        assert np.array_equal(idx.partition(), phi % idx.B)
+        if fold:  # documents that are there already and new ones, after the fold
+            insert(corpus.doc_ids[:K // 2])
+            _all_paths_match(rambo_lib, torch, idx, o, kmers, q)
