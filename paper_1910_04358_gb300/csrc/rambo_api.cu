@@ -1358,12 +1358,11 @@ int rambo_set_partition(rambo_t *h, const uint32_t *phi) {
         if (phi[i] >= h->g.B) return RAMBO_EINVAL;
     DeviceGuard guard(h->device);
     if (!guard.ok) return RAMBO_ECUDA;
+    // (on the handle's stream, which does not wait for the default stream: the
+    // patterns are made from the map behind its copy)
+    RAMBO_TRY(cudaMemcpyAsync(h->d_phi, phi, n * 4, cudaMemcpyHostToDevice, h->stream));
+    if (h->d_pattern) RAMBO_TRY(launch_patterns(h->g, h->d_pattern, h->d_phi, h->stream));
     RAMBO_TRY(cudaStreamSynchronize(h->stream));
-    RAMBO_TRY(cudaMemcpy(h->d_phi, phi, n * 4, cudaMemcpyHostToDevice));
-    if (h->d_pattern) {
-        RAMBO_TRY(launch_patterns(h->g, h->d_pattern, h->d_phi, h->stream));
-        RAMBO_TRY(cudaStreamSynchronize(h->stream));
-    }
     return RAMBO_OK;
 }
 

@@ -243,3 +243,22 @@ def test_fold_of_an_explicit_partition(rambo_lib, K, B, R):
         if fold:  # documents that are there already and new ones, after the fold
             insert(corpus.doc_ids[:K // 2])
             _all_paths_match(rambo_lib, torch, idx, o, kmers, q)
+
+
+def test_insertion_right_after_set_partition_uses_the_new_map(rambo_lib):
+    # the last documents of a map that takes a while to copy, inserted with one
+    # k-mer each: the only group that is set holds the new buckets and no other
+    K, B, R = 1 << 20, 32, 4
+    rng = np.random.default_rng(3)
+    packed, offs = synth.pack_many([synth.uniform_genome(rng, 15)] * 64)
+    ids = np.arange(K - 64, K, dtype=np.uint32)
+    for i in range(20):
+        phi = rng.integers(0, B, size=(K, R)).astype(np.uint32)
+        with rambo_lib.Index(K, B, R, 1 << 8, 1, 15, seed=i) as idx:
+            idx.set_partition(phi)
+            idx.insert_batch(ids, packed, offs)
+            rows = idx.copy_index().reshape(1 << 8, -1)
+        hit = np.nonzero(rows.any(axis=1))[0]
+        assert hit.size == 1, i
+        got = np.nonzero(np.unpackbits(rows[hit[0]], bitorder="little"))[0]
+        assert np.array_equal(got, np.unique(phi[ids] + B * np.arange(R, dtype=np.uint32))), i
