@@ -334,8 +334,13 @@ __global__ void __launch_bounds__(ANS_THREADS, 3) k_answers(AnswerArgs a) {
 template <int RT, int ETA, bool SHARED>
 cudaError_t launch_answers_t(AnswerArgs &a, int max_blocks, int sm_count, cudaStream_t s) {
     const size_t smem = ((size_t)ANS_WARPS * ANS_STAGE + (size_t)a.m_words * (SHARED ? 1 : ANS_WARPS)) * 4;
+    // (the limit belongs to the kernel, not to the launch: always the most that
+    // any geometry takes, so that launches of several threads don't lower one
+    // another's)
+    constexpr size_t limit = ((size_t)ANS_WARPS * ANS_STAGE + (SHARED ? ANS_MAX_SLOTS : ANS_WARPS * ANS_WARP_TABLE_MAX)) * 4;
+    if (smem > limit) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k_answers<RT, ETA, SHARED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         (int)limit);
     if (e != cudaSuccess) return e;
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_answers<RT, ETA, SHARED>, ANS_THREADS, smem);

@@ -403,9 +403,10 @@ cudaError_t launch_probe_pass(const BinnedArgs &a, int sm_count, cudaStream_t s)
 template <int SW>
 int scatter_blocks_per_sm(size_t smem) {
     // (always set: the kernel's static shared memory counts against the
-    // default 48 KB too)
-    if (cudaFuncSetAttribute(k_bin_scatter<SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    // default 48 KB too; and always to the most that any launch takes: the limit
+    // belongs to the kernel, and several threads must not lower one another's)
+    if (cudaFuncSetAttribute(k_bin_scatter<SW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)scatter_smem((uint32_t)BIN_MAX, BINNED_TILE_RECS)) != cudaSuccess)
         return 1;
     int occ = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bin_scatter<SW>, SCATTER_THREADS, smem) !=

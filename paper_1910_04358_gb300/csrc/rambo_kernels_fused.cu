@@ -351,7 +351,10 @@ cudaError_t launch_fused_t(const FusedArgs &f, int grid_override, int sm_count, 
     if (e != cudaSuccess) return e;
     const size_t hsmem = (size_t)HEAVY_WARPS * f.e.R * f.e.B * sizeof(uint16_t);
     if (hsmem > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_fused_heavy<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsmem);
+        // (the most that any launch takes, groups of 512 bytes: the limit belongs
+        // to the kernel, and several threads must not lower one another's)
+        e = cudaFuncSetAttribute(k_fused_heavy<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 HEAVY_WARPS * 512 * 8 * (int)sizeof(uint16_t));
         if (e != cudaSuccess) return e;
     }
     k_fused_heavy<C><<<sm_count * 4, HEAVY_WARPS * 32, hsmem, s>>>(f);

@@ -379,10 +379,12 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, B
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// (most: what any launch of the kernel takes; the limit belongs to the kernel,
+// so launches of several threads must not lower one another's)
 template <typename KernelT>
-int ib_blocks_per_sm(KernelT kernel, size_t smem) {
+int ib_blocks_per_sm(KernelT kernel, size_t smem, size_t most) {
     int n = 0;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, IB_THREADS, smem) != cudaSuccess || n < 1)
         n = 1;
     return n;
@@ -396,8 +398,8 @@ template <int ETA, int KIND>
 cudaError_t launch_scatter(const InsertArgs &a, const BinnedInsert &b, uint64_t f0, uint64_t f1, int sm_count,
                            cudaStream_t s) {
     const auto kernel = k_insert_bin_scatter<ETA, KIND>;
-    const int occ = ib_blocks_per_sm(kernel, scatter_smem());
-kernel<<<sm_count * occ * SCATTER_WAVES, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
+    const int occ = ib_blocks_per_sm(kernel, scatter_smem(), scatter_smem());
+    kernel<<<sm_count * occ * SCATTER_WAVES, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
     return cudaGetLastError();
 }
 
@@ -408,7 +410,7 @@ template <int KIND, bool SPAT>
 cudaError_t launch_apply(const InsertArgs &a, const BinnedInsert &b, int sm_count, cudaStream_t s) {
     const auto kernel = k_insert_bin_apply<KIND, SPAT>;
     const size_t smem = apply_smem(SPAT ? (size_t)a.K * a.lanes * 8 : 0);
-    const int occ = ib_blocks_per_sm(kernel, smem);
+    const int occ = ib_blocks_per_sm(kernel, smem, apply_smem(SPAT ? IB_PATTERN_MAX : 0));
     kernel<<<sm_count * occ, IB_THREADS, smem, s>>>(a, b);
     return cudaGetLastError();
 }

@@ -55,3 +55,37 @@ print(log().decode())
     copy, launch = [l for l in lines if l]
     assert copy.startswith("copy bytes=1600") and "k_patterns" in launch
     assert "stream=" in copy and _stream(copy) == _stream(launch)
+
+
+def test_shared_memory_limits_do_not_depend_on_the_handle(calls):
+    # a kernel's limit outlives the launch: a handle that sets it to its own size
+    # lowers it under another thread's launch
+    lines = calls("""
+from paper_1910_04358_gb300.rambo import load, _check
+for K, B, R in [(600, 27, 3), (200, 60, 3), (200, 500, 3), (90, 4000, 3), (300, 31, 4), (100, 32, 4), (60, 1000, 4), (60, 800, 5),
+                (60, 650, 5)]:
+    idx = rambo.Index(K, B, R, 1 << 12, 2, k=15)
+    log()
+    idx.set_tuning(insert_mode=3, bin_region_kib=1 + B // 100, early_exit=1)
+    ids, offs = np.arange(8, dtype=np.uint32), np.arange(9, dtype=np.uint64) * 100
+    idx.insert_batch(ids, np.zeros(300, np.uint8), offs)
+    idx.query_kmers(np.arange(50))
+    for path in (0, 1, 2):
+        idx.set_tuning(query_path=path)
+        idx.query_seqs(np.zeros(300, np.uint8), offs)
+    print(log().decode())
+    idx.close()
+""")
+    limits, launched = {}, {}
+    for line in lines:
+        w = line.split()
+        if line.startswith("limit "):
+            limits.setdefault(w[1], set()).add(int(w[2]))
+        elif line.startswith("launch "):
+            launched.setdefault(w[1], set()).add(int(re.search(r"smem=(\d+)", line).group(1)))
+    for kernel in ("k_answers", "k_insert_bin_apply", "k_insert_bin_scatter", "k_bin_scatter", "k_fused_heavy"):
+        assert any(kernel in k for k in limits), kernel
+    for kernel, values in limits.items():
+        assert len(values) == 1, (kernel, values)
+        assert max(values) >= max(launched.get(kernel, {0})) and max(values) <= 227 * 1024, kernel
+    assert any(len(v) > 1 for k, v in launched.items() if "k_answers" in k)
