@@ -91,9 +91,9 @@ template <int ETA>
 __host__ __device__ constexpr size_t fused_stage_bytes() { return (size_t)(FUSED_THREADS / 32) * probe_rif<1, ETA>() * ETA * 32 * 16; }
 
 template <int SW, int LPG, int ETA, int C, bool ASYNC>
-// three resident blocks per SM fit without spills for groups read by 4+
-// lanes; one-lane groups keep 16 loads per lane in flight at two (in
-// registers) or at three (staged in shared memory)
+// three resident blocks per SM for groups read by 4+ lanes (at the price of
+// spills of up to 76 bytes a thread); one-lane groups keep 16 loads per lane in
+// flight at two (in registers) or at three (staged in shared memory)
 __global__ void __launch_bounds__(FUSED_THREADS, (LPG >= 4 || ASYNC) ? 3 : 2) k_fused(FusedArgs f) {
     __shared__ uint32_t bm_smem[FUSED_THREADS / 32][128];
     __shared__ uint32_t list_smem[FUSED_THREADS / 32][EXPAND_LIST_MAX];
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, (LPG >= 4 || ASYNC) ? 3 : 2) k_
             const uint64_t seg = f.early_exit ? f.segment : (k1 > k0 ? k1 - k0 : 1);
             for (uint64_t a0 = k0; a0 < k1; a0 += seg) {
                 const uint64_t a1 = a0 + seg < k1 ? a0 + seg : k1;
-                slice_and(s, probe_range<SW, LPG, ETA, ASYNC, false>(f.p, start, a0, a1, lane, word0, stage));
+                slice_and(s, probe_counted<SW, LPG, ETA, ASYNC, false, (LPG >= 4)>(f.p, start, a0, a1, lane, word0, stage));
                 if (!f.early_exit) continue;
                 if (lane == 0 && f.probed) atomicAdd(f.probed, (unsigned long long)(a1 - a0));
                 if (a1 >= k1) break;
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, (LPG >= 4 || ASYNC) ? 3 : 2) k_
         const uint64_t seg = f.early_exit ? f.segment : (nk ? nk : 1);
         for (uint64_t k0 = 0; k0 < nk; k0 += seg) {
             const uint64_t k1 = k0 + seg < nk ? k0 + seg : nk;
-            slice_and(sl, probe_range<SW, LPG, ETA, ASYNC, false>(f.p, start, k0, k1, lane, word0, stage));
+            slice_and(sl, probe_counted<SW, LPG, ETA, ASYNC, false, (LPG >= 4)>(f.p, start, k0, k1, lane, word0, stage));
             if (!f.early_exit) continue;
             if (lane == 0 && f.probed) atomicAdd(f.probed, (unsigned long long)(k1 - k0));
             if (k1 >= nk) break;

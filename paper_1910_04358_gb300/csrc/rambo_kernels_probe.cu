@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(PROBE_THREADS, LPG == 1 ? 2 : 3) k_probe_tiles
         }
         const uint64_t b0 = a.offsets[q], nk = a.ends[q] - b0 - a.k + 1;  // (a query with tiles has k-mers)
         const uint64_t k0 = (t - first) * tile, k1 = k0 + tile < nk ? k0 + tile : nk;
-        const Slice<SW> s = probe_range<SW, LPG, ETA, false, true>(a, b0, k0, k1, lane, word0, nullptr);
+        const Slice<SW> s = probe_counted<SW, LPG, ETA, false, true, LPG == 4>(a, b0, k0, k1, lane, word0, nullptr);
         if (lane < LPG) {
             if (next - first == 1) {
                 uint32_t *p = a.acc + q * a.Gw + word0;

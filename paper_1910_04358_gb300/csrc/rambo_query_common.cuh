@@ -77,15 +77,15 @@ __device__ __forceinline__ void flush_slice(uint32_t *acc, uint64_t q, uint32_t 
 template <int LPG, int ETA>
 __host__ __device__ constexpr int probe_rif() { return (LPG == 1 ? 8 : 4) / (ETA <= 2 ? 1 : 2); }
 
-// AND of the groups of k-mers [k0, k1) of one query, per lane slice (every
-// lane of the warp works on the same query).  ASYNC (one lane per 16-byte
-// group): the gathers land in the warp's shared-memory `stage` through
+// AND of the groups of k-mers [k0, k1) of the stretch at base `start`, per lane
+// slice (every lane of the warp works on the same query).  ASYNC (one lane per
+// 16-byte group): the gathers land in the warp's shared-memory `stage` through
 // cp.async instead of registers, so a lane holds no load data in flight.
 // SKIP: tiles of 32 k-mers past the end are not hashed (short ranges).
-template <int SW, int LPG, int ETA, bool ASYNC, bool SKIP>
-__device__ __forceinline__ Slice<SW> probe_range(const ProbeArgs &a, uint64_t start,
-                                                        uint64_t k0, uint64_t k1, int lane,
-                                                        uint32_t word0, uint4 *stage) {
+// N: the type that counts them (k1 at most 2^30).
+template <int SW, int LPG, int ETA, bool ASYNC, bool SKIP, typename N>
+__device__ __forceinline__ Slice<SW> probe_range(const ProbeArgs &a, uint64_t start, N k0, N k1, int lane,
+                                                 uint32_t word0, uint4 *stage) {
     static_assert(!ASYNC || (LPG == 1 && SW == 4), "staged gathers: one lane per 16-byte group");
     constexpr int RIF = probe_rif<LPG, ETA>();  // rounds whose loads are in flight together
     constexpr int NT = LPG >= RIF ? 1 : RIF / LPG;
@@ -96,14 +96,14 @@ __device__ __forceinline__ Slice<SW> probe_range(const ProbeArgs &a, uint64_t st
     Slice<SW> accv;
     slice_ones(accv);
     for (uint32_t jb = 0; jb < a.eta; jb += ETA) {
-        for (uint64_t base = k0; base < k1; base += STEP) {
+        for (N base = k0; base < k1; base += STEP) {
             uint32_t pos[NT][ETA];
             bool val[NT];
 #pragma unroll
             for (int t = 0; t < NT; ++t) {
-                const uint64_t g = base + (uint64_t)t * 32 + lane;
+                const N g = base + t * 32 + lane;
                 val[t] = g < k1;
-                if (SKIP && t > 0 && base + (uint64_t)t * 32 >= k1) continue;  // the whole warp
+                if (SKIP && t > 0 && base + t * 32 >= k1) continue;  // the whole warp
                 uint64_t c = 0;
                 if (val[t])
                     c = canonical_from_window(base_window(a.packed, a.packed_bytes, start + a.base_shift + g), a.k);
@@ -169,6 +169,18 @@ __device__ __forceinline__ Slice<SW> probe_range(const ProbeArgs &a, uint64_t st
 #pragma unroll
         for (int off = LPG; off < 32; off <<= 1) accv.w[w] &= __shfl_xor_sync(FULL, accv.w[w], off);
     return accv;
+}
+
+// probe_range counting in 64 or 32 bits (k1 - k0 at most 2^30).  32 take fewer
+// registers: 16-byte groups in the separate launch 2% faster, and no spills in
+// the persistent one.  But on 64-byte groups both are 1-2% slower with them, and
+// the persistent launch on wider ones spills more and is 4-6% slower.
+template <int SW, int LPG, int ETA, bool ASYNC, bool SKIP, bool COUNT64>
+__device__ __forceinline__ Slice<SW> probe_counted(const ProbeArgs &a, uint64_t start, uint64_t k0, uint64_t k1, int lane,
+                                                   uint32_t word0, uint4 *stage) {
+    if constexpr (COUNT64) return probe_range<SW, LPG, ETA, ASYNC, SKIP, uint64_t>(a, start, k0, k1, lane, word0, stage);
+    else
+        return probe_range<SW, LPG, ETA, ASYNC, SKIP, uint32_t>(a, start + k0, 0, (uint32_t)(k1 - k0), lane, word0, stage);
 }
 
 // Per-warp contiguous range of the flattened k-mer index space [0, T).
