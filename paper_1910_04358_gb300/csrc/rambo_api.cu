@@ -542,7 +542,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
         RAMBO_TRY(launch_fused(a, e, g, qs, go, h->sm_count, s));
         return RAMBO_OK;
     }
-    const uint32_t tile = probe_tile_kmers(packed_bytes * 4, h->sm_count);
+    const uint32_t tile = probe_tile_kmers(n, packed_bytes * 4, h->sm_count);
     {
         StageScope sc(h, RAMBO_STAGE_PREFIX, s, kmer_prefix_launches(n));
         RAMBO_TRY(launch_kmer_prefix(offsets, ends, n, g.k, packed_bytes, kcum, bsum, h->d_err, s, tile, 0, acc,
@@ -567,6 +567,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
     a.err = h->d_err;
     a.min_chunk = h->tune.probe_min_kmers_per_warp;
     a.max_kmers = packed_bytes * 4;
+    a.few = probe_few_items(n, packed_bytes * 4, h->sm_count);
     {
         StageScope sc(h, RAMBO_STAGE_PROBE_SEQS, s, 1);
         RAMBO_TRY(launch_probe_seqs(a, g, tile, probe_grid(h), s));

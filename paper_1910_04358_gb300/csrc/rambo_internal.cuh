@@ -199,6 +199,7 @@ struct ProbeArgs {
     uint32_t *err;
     uint32_t min_chunk;      // minimum k-mers per warp (0 = default)
     uint64_t max_kmers;      // sequence batch: about how many k-mers it has (grid sizing only)
+    uint32_t few;            // separate probe launch: probe_few_items
 };
 
 struct ExpandArgs {
@@ -304,8 +305,14 @@ cudaError_t launch_fold(const uint32_t *old_index, uint32_t old_gw, uint32_t *ne
                         uint32_t new_gw, uint64_t m, uint32_t B, uint32_t R,
                         const uint32_t *old_db, uint32_t *new_db, uint32_t W, int sm_count,
                         cudaStream_t s);
-// k-mers per tile for a batch of about max_kmers k-mers
-uint32_t probe_tile_kmers(uint64_t max_kmers, int sm_count);
+// A batch of few items over many bases, n and max_kmers as the launch knows
+// them: tiles of an even share would leave one round of warps full and the next
+// nearly empty (2,000 items of 1,000 k-mers, 512-byte groups: 411 us against
+// 333), and a few places in a large buffer would be cut as if they were all of
+// it.  Their tiles are small, and warps take several.
+bool probe_few_items(uint64_t n, uint64_t max_kmers, int sm_count);
+// k-mers per tile of a batch of n items in a buffer of max_kmers k-mers
+uint32_t probe_tile_kmers(uint64_t n, uint64_t max_kmers, int sm_count);
 // kcum: the batch's tile prefix (launch_kmer_prefix, `tile`); acc set to ones
 cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm_count, cudaStream_t s);
 // (groups of 512 bytes and more; the others are probed by launch_kmer_answers)

@@ -18,26 +18,46 @@ namespace {
 // slice (16 bytes when the group is >= 16 bytes), so one warp instruction
 // reads 32/LPG whole groups as runs of full 32-byte sectors (probe_range).
 // The batch is cut into tiles of at most `tile` k-mers of one query, numbered
-// by a prefix scan (kcum); every warp takes `per` consecutive tiles, ANDs a
-// tile's groups over its lanes and writes one mask: a plain store when the
-// query is a single tile, else an atomicAnd into the mask set to ones.  Bound
-// by the DRAM lines of the gathers (128 bytes each, whatever the group).
-// A warp that walked k-mers regardless of their query had every lane flush
-// its own slice at each query's end, 128 atomics for a 32-byte group.
-template <int SW, int LPG, int ETA>
-__global__ void __launch_bounds__(PROBE_THREADS, LPG == 1 ? 2 : 3) k_probe_tiles(ProbeArgs a, uint32_t tile, uint32_t per) {
+// by a prefix scan (kcum); every warp takes consecutive tiles, ANDs a tile's
+// groups over its lanes and writes one mask: a plain store when the query is a
+// single tile, else an atomicAnd into the mask set to ones.  Bound by the DRAM
+// lines of the gathers (128 bytes each, whatever the group).  A warp that
+// walked k-mers regardless of their query had every lane flush its own slice at
+// each query's end, 128 atomics for a 32-byte group.
+// FEW (probe_few_items: small tiles): a query's tiles are ANDed together in shared
+// memory first, one atomicAnd for all of a warp's (one for every tile of 128
+// k-mers doubles the time of a single sequence of 3*10^7 bases).  A template of
+// its own: the state it keeps costs the other batches 2-5% on groups of 64 and
+// 128 bytes, whose instances are short of registers.
+struct TileShare {
+    uint32_t tile;      // k-mers
+    uint32_t per;       // tiles a warp takes, at most, unless the warps would not cover the batch
+    uint32_t resident;  // warps that are resident together
+};
+
+// FEW: shares that every resident warp gets before they grow past one tile.
+constexpr uint32_t FEW_ROUNDS = 4;
+
+template <int SW, int LPG, int ETA, bool FEW>
+__global__ void __launch_bounds__(PROBE_THREADS, LPG == 1 ? 2 : 3) k_probe_tiles(ProbeArgs a, TileShare sh) {
+    __shared__ uint32_t run_smem[FEW ? PROBE_THREADS / 32 : 1][LPG * SW];  // a query's mask over the warp's tiles
     const int lane = threadIdx.x & 31;
     const uint32_t word0 = blockIdx.y * (LPG * SW) + (lane % LPG) * SW;
     const uint64_t tiles = a.kcum[a.n];
     const uint64_t warp = (uint64_t)blockIdx.x * (PROBE_THREADS / 32) + (threadIdx.x >> 5);
     const uint64_t nwarps = (uint64_t)gridDim.x * (PROBE_THREADS / 32);
-    // (`per` comes from the bases the batch is known to span; items that overlap
-    // have more tiles, which the warps then share evenly)
-    const uint64_t even = (tiles + nwarps - 1) / nwarps;
-    const uint64_t mine = per > even ? per : even;
+    // (The launch knows only the bases that the batch's buffer spans: items may
+    // overlap and have more tiles, or be a few places in it and have far fewer.)
+    const uint64_t busy = tiles / (FEW ? FEW_ROUNDS * sh.resident : sh.resident), even = (tiles + nwarps - 1) / nwarps;
+    uint64_t mine = sh.per < busy ? sh.per : busy;
+    if (mine < even) mine = even;
     const uint64_t t0 = warp * mine;
     if (t0 >= tiles) return;
     const uint64_t t1 = t0 + mine < tiles ? t0 + mine : tiles;
+    // (each lane that holds a mask, the first LPG, has its words to itself)
+    if (FEW && LPG >= 8 && lane < LPG)
+#pragma unroll
+        for (int w = 0; w < SW; ++w) run_smem[threadIdx.x >> 5][lane * SW + w] = FULL;
     uint64_t q = find_query_warp(a.kcum, a.n, t0, lane);
     uint64_t first = a.kcum[q], next = a.kcum[q + 1];
     for (uint64_t t = t0; t < t1; ++t) {
@@ -47,19 +67,30 @@ __global__ void __launch_bounds__(PROBE_THREADS, LPG == 1 ? 2 : 3) k_probe_tiles
             next = a.kcum[q + 1];
         }
         const uint64_t b0 = a.offsets[q], nk = a.ends[q] - b0 - a.k + 1;  // (a query with tiles has k-mers)
-        const uint64_t k0 = (t - first) * tile, k1 = k0 + tile < nk ? k0 + tile : nk;
-        const Slice<SW> s = probe_counted<SW, LPG, ETA, false, true, LPG == 4>(a, b0, k0, k1, lane, word0, nullptr);
-        if (lane < LPG) {
-            if (next - first == 1) {
-                uint32_t *p = a.acc + q * a.Gw + word0;
-                if constexpr (SW == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(s.w[0], s.w[1], s.w[2], s.w[3]);
-                else
+        const uint64_t k0 = (t - first) * sh.tile, k1 = k0 + sh.tile < nk ? k0 + sh.tile : nk;
+        Slice<SW> s = probe_counted<SW, LPG, ETA, false, true, LPG == 4>(a, b0, k0, k1, lane, word0, nullptr);
+        if (lane >= LPG) continue;
+        if (next - first == 1) {
+            uint32_t *p = a.acc + q * a.Gw + word0;
+            if constexpr (SW == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(s.w[0], s.w[1], s.w[2], s.w[3]);
+            else
 #pragma unroll
-                    for (int w = 0; w < SW; ++w) p[w] = s.w[w];
-            } else {
-                flush_slice<SW>(a.acc, q, a.Gw, word0, s);
-            }
+                for (int w = 0; w < SW; ++w) p[w] = s.w[w];
+            continue;
         }
+        if constexpr (FEW) {
+            // (before a query's first tile the wide instances hold ones, the
+            // others skip the words: the form that spills least)
+            uint32_t *run = run_smem[threadIdx.x >> 5] + lane * SW;
+            const bool ends = t + 1 == t1 || t + 1 == next;
+            if (LPG >= 8 || (t != t0 && t != first))
+#pragma unroll
+                for (int w = 0; w < SW; ++w) s.w[w] &= run[w];
+#pragma unroll
+            for (int w = 0; w < SW; ++w) run[w] = LPG >= 8 && ends ? FULL : s.w[w];
+            if (!ends) continue;
+        }
+        flush_slice<SW>(a.acc, q, a.Gw, word0, s);
     }
 }
 
@@ -153,31 +184,39 @@ __global__ void __launch_bounds__(PROBE_THREADS) k_probe_kmers(ProbeArgs a) {
 // with 4,096 k-mers a warp, 10.27 with 512 and 10.26 with 256; 20,000 short
 // reads 170, 170, 155 and 148 us.
 constexpr uint64_t SEQ_SHARE = 256;
-
-// K-mers per tile of a batch of about max_kmers k-mers: 1,024 (of 16 or more
-// rounds of loads), fewer when that leaves warps without a tile.
-uint32_t tile_kmers(uint64_t max_kmers, int sm_count) {
-    uint64_t t = max_kmers / ((uint64_t)sm_count * 24);
-    t = t / 64 * 64;
-    return (uint32_t)(t < 128 ? 128 : t > 1024 ? 1024 : t);
-}
+// Warps that are resident on an SM.
+constexpr uint32_t SEQ_RESIDENT = 24;
+// Most blocks for every resident one, which leaves a warp 4,000 k-mers and more
+// of a batch that has them: where a batch is a few places in its buffer, every
+// further block finds nothing to do (500 ranges of 1,000 k-mers in 1.25 GB,
+// 64-byte groups: 540 us with a block for every 8,192 bases of the buffer, 62
+// like this).
+constexpr uint64_t SEQ_WAVES = 16;
+constexpr uint32_t SEQ_TILE = 128, SEQ_TILE_MAX = 1024;
 
 // sm_count > 0: sized by the batch; sm_count < 0: -sm_count CTAs
 template <int SW, int LPG, int ETA>
 cudaError_t launch_seqs_t(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm_count, cudaStream_t s) {
     constexpr uint64_t WARPS = PROBE_THREADS / 32;
     uint64_t blocks = (uint64_t)-(int64_t)sm_count;
-    uint32_t per = 0;
+    TileShare sh{tile, 0, 1};
+    const bool few = a.few != 0;
     if (sm_count > 0) {
+        sh.resident = (uint32_t)sm_count * SEQ_RESIDENT;
         const uint64_t tiles = a.n + a.max_kmers / tile;  // at least as many as items that do not overlap have
-        uint64_t share = a.min_chunk > SEQ_SHARE ? a.min_chunk : SEQ_SHARE;
-        uint64_t want = share * tiles / (a.max_kmers ? a.max_kmers : 1);
-        const uint64_t most = tiles / ((uint64_t)sm_count * 24);  // keep every warp busy first
+        uint64_t share = few ? SEQ_TILE_MAX : SEQ_SHARE;
+        if (share < a.min_chunk) share = a.min_chunk;
+        uint64_t want = few ? share / SEQ_TILE : share * tiles / (a.max_kmers ? a.max_kmers : 1);
+        const uint64_t most = tiles / (few ? FEW_ROUNDS * sh.resident : sh.resident);  // keep every warp busy first
         if (want > most) want = most;
-        per = want < 1 ? 1 : want > 1024 ? 1024 : (uint32_t)want;
-        blocks = (tiles + WARPS * per - 1) / (WARPS * per);
+        sh.per = want < 1 ? 1 : want > 1024 ? 1024 : (uint32_t)want;
+        blocks = (tiles + WARPS * sh.per - 1) / (WARPS * sh.per);
+        const uint64_t cap = sh.resident / WARPS * SEQ_WAVES;
+        if (blocks > cap) blocks = cap;
     }
-    k_probe_tiles<SW, LPG, ETA><<<dim3((unsigned)blocks, g.chunks), PROBE_THREADS, 0, s>>>(a, tile, per);
+    const dim3 grid((unsigned)blocks, g.chunks);
+    if (few) k_probe_tiles<SW, LPG, ETA, true><<<grid, PROBE_THREADS, 0, s>>>(a, sh);
+    else k_probe_tiles<SW, LPG, ETA, false><<<grid, PROBE_THREADS, 0, s>>>(a, sh);
     return cudaGetLastError();
 }
 
@@ -201,7 +240,22 @@ cudaError_t launch_kmers_t(const ProbeArgs &a, const Geometry &g, int sm_count, 
 
 }  // namespace
 
-uint32_t probe_tile_kmers(uint64_t max_kmers, int sm_count) { return tile_kmers(max_kmers, sm_count); }
+// Twice the resident warps: with more items, one tile each fills the rounds
+// (10,000 of 1,000 k-mers, 128-byte groups: 446 us, 468 with small tiles; 8,000
+// of them 394 and 397).  512 k-mers a warp: with fewer, tiles of an even share
+// are small already.
+bool probe_few_items(uint64_t n, uint64_t max_kmers, int sm_count) {
+    const uint64_t warps = (uint64_t)sm_count * SEQ_RESIDENT;
+    return n < 2 * warps && max_kmers >= 512 * warps;
+}
+
+// 1,024 (of 16 or more rounds of loads), fewer when that leaves warps without
+// a tile.
+uint32_t probe_tile_kmers(uint64_t n, uint64_t max_kmers, int sm_count) {
+    if (probe_few_items(n, max_kmers, sm_count)) return SEQ_TILE;
+    const uint64_t t = max_kmers / ((uint64_t)sm_count * SEQ_RESIDENT) / 64 * 64;
+    return (uint32_t)(t < SEQ_TILE ? SEQ_TILE : t > SEQ_TILE_MAX ? SEQ_TILE_MAX : t);
+}
 
 cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm_count, cudaStream_t s) {
     if (g.SW == 1) return launch_seqs_eta<1, 1>(a, g, tile, sm_count, s);

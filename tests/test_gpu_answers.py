@@ -262,3 +262,42 @@ def test_insertion_right_after_set_partition_uses_the_new_map(rambo_lib):
         assert hit.size == 1, i
         got = np.nonzero(np.unpackbits(rows[hit[0]], bitorder="little"))[0]
         assert np.array_equal(got, np.unique(phi[ids] + B * np.arange(R, dtype=np.uint32))), i
+
+
+@pytest.mark.parametrize("B,R", [(10, 3), (32, 4), (60, 4), (100, 5), (200, 5), (400, 6), (500, 8), (600, 8)])
+def test_few_items_in_a_large_buffer(rambo_lib, B, R):
+    # fewer items than resident warps over bases for 512 k-mers a warp and more:
+    # tiles of 128 k-mers, a query's tiles of one warp in one mask.  A few ranges
+    # of the buffer, items that cover it (of some tiles, and of thousands), and
+    # the same with a fixed grid, whose warps take many tiles.
+    import torch
+    p = synth.Params(K=70, B=B, R=R, m=(1 << 14) + 5, eta=2, k=31, seed=5)
+    rng = np.random.default_rng(B)
+    corpus = synth.family_corpus(rng, p, n_seeds=6, doc_len=4000, sub_rate=0.001)
+    o = oracle.Rambo(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    idx = rambo_lib.Index(p.K, p.B, p.R, p.m, p.eta, p.k, p.seed)
+    for x in (o, idx):
+        x.insert_batch(corpus.doc_ids, corpus.packed, corpus.offsets)
+    total = 152 * 24 * 512 + 4001
+    bases = synth.uniform_genome(rng, total)
+    at = np.arange(0, total - 4100, 6000)
+    for i, a in enumerate(at):  # documents here and there, random bases between
+        bases[a:a + 4000] = corpus.doc_bases(i % p.K)
+    packed = synth.pack_bases(bases)
+    few = np.sort(rng.choice(at, 40, replace=False))
+    cases = [(few, few + rng.choice([20, 31, 157, 158, 159, 1000, 4000], size=40)),
+             (np.arange(0, total, 2500), np.append(np.arange(2500, total, 2500), total)),
+             (np.array([0, 9, 1000]), np.array([9, 1000, total]))]
+    dp = _dev(torch, np.concatenate([packed, np.zeros(16, np.uint8)]), np.uint8)
+    hits = 0
+    for begins, ends in cases:
+        qp, qo = synth.pack_many([bases[b:e] for b, e in zip(begins, ends)])
+        want = o.query_seqs(qp, qo, threads=4)
+        hits += np.count_nonzero(want)
+        for ctas in (0, 1):
+            idx.set_tuning(query_path=0, probe_ctas_per_sm=ctas)
+            got = idx.query_ranges_dev(dp, _dev(torch, begins.astype(np.int64), np.int64),
+                                       _dev(torch, ends.astype(np.int64), np.int64))
+            idx.sync()
+            assert np.array_equal(rambo_lib.as_u32(got), want), (len(begins), ctas)
+    assert hits > 40

@@ -89,3 +89,23 @@ for K, B, R in [(600, 27, 3), (200, 60, 3), (200, 500, 3), (90, 4000, 3), (300, 
         assert len(values) == 1, (kernel, values)
         assert max(values) >= max(launched.get(kernel, {0})) and max(values) <= 227 * 1024, kernel
     assert any(len(v) > 1 for k, v in launched.items() if "k_answers" in k)
+
+
+def test_sequence_probe_grid_of_a_few_ranges_of_a_large_buffer(calls):
+    # blocks for every base of the buffer would nearly all find nothing to do
+    lines = calls("""
+idx = rambo.Index(100, 100, 5, 256, 2)
+L = rambo.load()
+z = np.zeros(10, np.uint8)
+for n, nbytes in [(500, 1_250_000_000), (5000, 1_250_000_000), (256, 30_080), (20_000, 850_000)]:
+    b = np.zeros(n + 1, np.uint64)
+    out, ws = np.zeros((n, idx.W), np.uint32), aligned(idx.workspace_bytes("seqs", n))
+    log()
+    rambo._check(L.rambo_query_ranges_dev(idx._h, n, ptr(z), nbytes, ptr(b), ptr(b) + 8, ptr(out), ptr(ws), ws.size, None), "q")
+    print([l for l in log().decode().splitlines() if "k_probe_tiles" in l][0])
+""")
+    blocks = [int(re.search(r"grid=(\d+),1 ", line).group(1)) for line in lines]
+    resident = 152 * 3
+    assert resident <= blocks[0] <= 16 * resident and resident <= blocks[1] <= 16 * resident
+    assert 120 <= blocks[2] <= 256           # a warp for every 128 k-mers
+    assert 2000 <= blocks[3] <= 3500         # about a warp a read
