@@ -491,14 +491,24 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
     // The separate launches serve path 1 too where they are the faster ones: a
     // batch of less than a tile per resident warp, which leaves the persistent
     // launch short of work (256 requests of 470 bases: 24 against 253 us), and
-    // one-lane groups, unless the launch has to leave room for k-mer chunks
-    // (10^4 x 1 kbp beside 10^6 k-mers: 460 against 489 us; the same call with
-    // host buffers 0.88 against 0.80 ms).  Wider groups keep the persistent
-    // launch, which hides the expansion under the gathers (streaming epoch,
-    // 12.5 KB answers: 0.85 against 0.93 ms; 32 GiB index: equal).
+    // one-lane groups (16 bytes: 10^4 sequences of 1 kbp 470 against 479 us,
+    // 20,000 of 170 bases 158 against 205), unless the launch has to leave room
+    // for k-mer chunks (10^4 x 1 kbp beside 10^6 k-mers: 460 against 489 us; the
+    // same call with host buffers 0.88 against 0.80 ms).  Wider groups keep the
+    // persistent launch, which hides the expansion under the gathers (streaming
+    // epoch, 12.5 KB answers: 0.85 against 0.93 ms; 32 GiB index: equal).
     const bool one_lane = g.LPG == 1 && fused_ctas_cap == 0;
     const bool small = packed_bytes * 4 < (uint64_t)h->sm_count * 24 * h->tune.fused_tile_kmers;
-    const bool separate = !h->tune.early_exit && (one_lane || small);
+    // Answers of several chunks without a byte table cost the persistent launch
+    // little (it decodes a query's few buckets once).  From 16 queries an SM on it
+    // keeps two kinds of them: of a number of repetitions that the answer kernels
+    // don't unroll (40,000 documents, R = 8, 256-byte groups: 10,000 reads of 170
+    // bases 184 against 232 us, 2,000 sequences of 1 kbp 211 against 210), and of
+    // one-lane groups with queries long enough to hide them (200,000 documents:
+    // 10,000 of 1 kbp 495 against 564 us, of 170 bases 278 against 233).
+    const bool wide_lists = !h->d_tab && g.W > 128 && n >= (uint64_t)h->sm_count * 16;
+    const bool hidden = wide_lists && (g.R < 2 || g.R > 6 || (one_lane && packed_bytes * 4 >= 512 * n));
+    const bool separate = !h->tune.early_exit && (one_lane || small) && !hidden;
     if (h->tune.query_path >= 1 && !separate && fused_supported(g)) {
         // persistent fused query: length-bucketed queues, probe + expand in one launch
         ProbeArgs a{};

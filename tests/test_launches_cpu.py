@@ -109,3 +109,22 @@ for n, nbytes in [(500, 1_250_000_000), (5000, 1_250_000_000), (256, 30_080), (2
     assert resident <= blocks[0] <= 16 * resident and resident <= blocks[1] <= 16 * resident
     assert 120 <= blocks[2] <= 256           # a warp for every 128 k-mers
     assert 2000 <= blocks[3] <= 3500         # about a warp a read
+
+
+def test_path_1_keeps_the_persistent_launch_for_wide_answers_without_a_byte_table(calls):
+    lines = calls("""
+L = rambo.load()
+z = np.zeros(10, np.uint8)
+for K, B, R, tab, n, bases in [(40_000, 250, 8, 1, 3000, 170), (40_000, 250, 8, 1, 2000, 170), (40_000, 250, 6, 1, 3000, 170),
+                               (4000, 250, 8, 1, 3000, 170), (5000, 32, 4, 0, 3000, 1000), (5000, 32, 4, 0, 3000, 170),
+                               (5000, 32, 4, 1, 3000, 1000)]:
+    idx = rambo.Index(K, B, R, 256, 2)
+    idx.set_tuning(query_path=1, use_byte_table=tab)
+    b = np.zeros(n + 1, np.uint64)
+    out, ws = np.zeros((n, idx.W), np.uint32), aligned(idx.workspace_bytes("seqs", n))
+    log()
+    rambo._check(L.rambo_query_seqs_dev(idx._h, n, ptr(z), n * bases // 4, ptr(b), ptr(out), ptr(ws), ws.size, None), "q")
+    print("k_fused" in log().decode())
+    idx.close()
+""")
+    assert lines == ["True", "False", "False", "False", "True", "False", "False"]
