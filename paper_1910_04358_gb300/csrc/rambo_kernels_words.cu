@@ -90,45 +90,82 @@ __global__ void k_insert_words(WordArgs a) {
     }
 }
 
-// Probe of word queries: one warp per (query, term).  Lane j hashes the term
-// with seed j, then the lanes read the eta groups side by side, 16 bytes (or
-// a word) each, and fold their AND into the query's bucket mask with atomicAnd
-// (all-ones words skipped).  Bound by latency: 1,000 queries of 1..4 words on
-// 256-byte groups take 7 us, 34 with a thread per term walking the words.
+// Probe of word queries.  A term's L lanes hash it, lane j with seed j, then
+// read the eta groups side by side, 16 bytes (or a word) each, and fold their AND
+// into the query's bucket mask with atomicAnd (all-ones words skipped).
+// Up to a term a warp (9,728 on 152 SMs) the launch is bound by latency and a
+// term takes its whole warp, which finds the term's query together: 1,000
+// queries of 1..4 words on 256-byte groups 8 us, 33 with a thread per term.
+// Past that the warps go round, and a term takes only the lanes that have a seed
+// or a piece of the group (25,000 terms on 16-byte groups 10 us, 21 with a warp
+// each, 12 with a thread).  Past WORD_ROUNDS terms a warp a thread per term,
+// which needs no exchange, is the fastest (10^6 terms on 16-byte groups 62 us,
+// 81 with two lanes each, 630 with a warp), on groups of 256 bytes and more from
+// four times as many on (250,000 terms 154 us with lanes, 176 with threads;
+// 10^6 597 and 542).
 constexpr int WORD_THREADS = 256;
+constexpr uint64_t WORD_ROUNDS = 8;
+// A thread per term.
+__global__ void __launch_bounds__(WORD_THREADS) k_probe_words_by_thread(WordArgs a) {
+    const uint64_t t0 = a.item_terms[0], t1 = a.item_terms[a.n];
+    for (uint64_t t = t0 + (uint64_t)blockIdx.x * WORD_THREADS + threadIdx.x; t < t1; t += (uint64_t)gridDim.x * WORD_THREADS) {
+        const uint64_t q = item_of(a.item_terms, a.n, t);
+        const uint8_t *w;
+        uint64_t len;
+        if (!term_bytes(a, t, &w, &len)) continue;
+        uint32_t pos[64];
+        for (uint32_t j = 0; j < a.eta; ++j) pos[j] = reduce_pos(mh_bytes_first_word(w, len, a.seed32 + j), a.m, a.m_inv);
+        uint32_t *acc = a.acc + q * a.Gw;
+        for (uint32_t word = 0; word < a.Gw; ++word) {
+            uint32_t v = FULL;
+            for (uint32_t j = 0; j < a.eta && v; ++j) v &= __ldg(a.index_ro + (uint64_t)pos[j] * a.Gw + word);
+            if (v != FULL) atomicAnd(acc + word, v);
+        }
+    }
+}
 
-__global__ void __launch_bounds__(WORD_THREADS) k_probe_words(WordArgs a) {
+// `lanes` (a power of two) of a warp per term, or the warp.
+__global__ void __launch_bounds__(WORD_THREADS) k_probe_words(WordArgs a, uint32_t lanes) {
     const int lane = threadIdx.x & 31;
     const uint64_t t0 = a.item_terms[0], t1 = a.item_terms[a.n];
     const uint64_t nwarps = (uint64_t)gridDim.x * (WORD_THREADS / 32);
-    for (uint64_t t = t0 + (uint64_t)blockIdx.x * (WORD_THREADS / 32) + (threadIdx.x >> 5); t < t1; t += nwarps) {
-        const uint64_t q = find_query_warp(a.item_terms, a.n, t, lane);
+    const uint32_t L = t1 > t0 && t1 - t0 > nwarps ? lanes : 32;
+    const uint32_t per = 32 / L, mine = lane & (L - 1), lead = lane - mine;
+    const uint32_t pieces = (a.Gw & 3) == 0 ? a.Gw / 4 : a.Gw;  // of 16 bytes; groups of 4 or 8 bytes: words
+    for (uint64_t tb = t0 + ((uint64_t)blockIdx.x * (WORD_THREADS / 32) + (threadIdx.x >> 5)) * per; tb < t1;
+         tb += nwarps * per) {
+        const uint64_t t = tb + lead / L;
         const uint8_t *w = nullptr;
         uint64_t len = 0;
-        if (!term_bytes(a, t, &w, &len)) continue;  // the whole warp
+        bool live = t < t1;
+        uint64_t q = 0;
+        if (L == 32) q = find_query_warp(a.item_terms, a.n, t, lane);
+        else if (live) q = item_of(a.item_terms, a.n, t);
+        live = live && term_bytes(a, t, &w, &len);
         uint32_t *acc = a.acc + q * a.Gw;
-        for (uint32_t jb = 0; jb < a.eta; jb += 32) {
-            const uint32_t nj = a.eta - jb < 32 ? a.eta - jb : 32;
+        for (uint32_t jb = 0; jb < a.eta; jb += L) {
+            const uint32_t nj = a.eta - jb < L ? a.eta - jb : L;
             uint32_t pos = 0;
-            if ((uint32_t)lane < nj) pos = reduce_pos(mh_bytes_first_word(w, len, a.seed32 + jb + lane), a.m, a.m_inv);
-            if ((a.Gw & 3) == 0) {
-                for (uint32_t c0 = 0; c0 < a.Gw / 4; c0 += 32) {
-                    const uint32_t c = c0 + lane;
+            if (live && mine < nj) pos = reduce_pos(mh_bytes_first_word(w, len, a.seed32 + jb + mine), a.m, a.m_inv);
+            for (uint32_t c0 = 0; c0 < pieces; c0 += L) {
+                const uint32_t c = c0 + mine;
+                const bool reads = live && c < pieces;
+                if ((a.Gw & 3) == 0) {
                     Slice<4> v;
                     slice_ones(v);
                     for (uint32_t j = 0; j < nj; ++j) {
-                        const uint64_t p = __shfl_sync(FULL, pos, j);
-                        if (c < a.Gw / 4) slice_and(v, ld_slice<4>(a.index_ro + p * a.Gw + 4 * c));
+                        const uint64_t p = __shfl_sync(FULL, pos, lead + j);
+                        if (reads) slice_and(v, ld_slice<4>(a.index_ro + p * a.Gw + 4 * c));
                     }
-                    if (c < a.Gw / 4) flush_slice<4>(acc, 0, a.Gw, 4 * c, v);
+                    if (reads) flush_slice<4>(acc, 0, a.Gw, 4 * c, v);
+                } else {
+                    uint32_t v = FULL;
+                    for (uint32_t j = 0; j < nj; ++j) {
+                        const uint64_t p = __shfl_sync(FULL, pos, lead + j);
+                        if (reads) v &= __ldg(a.index_ro + p * a.Gw + c);
+                    }
+                    if (reads && v != FULL) atomicAnd(acc + c, v);
                 }
-            } else {  // groups of 4 or 8 bytes
-                uint32_t v = FULL;
-                for (uint32_t j = 0; j < nj; ++j) {
-                    const uint64_t p = __shfl_sync(FULL, pos, j);
-                    if ((uint32_t)lane < a.Gw) v &= __ldg(a.index_ro + p * a.Gw + lane);
-                }
-                if ((uint32_t)lane < a.Gw && v != FULL) atomicAnd(acc + lane, v);
             }
         }
     }
@@ -144,7 +181,18 @@ cudaError_t launch_insert_words(const WordArgs &a, int sm_count, cudaStream_t s)
 
 cudaError_t launch_probe_words(const WordArgs &a, int sm_count, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
-    k_probe_words<<<sm_count * 8, WORD_THREADS, 0, s>>>(a);
+    const uint32_t pieces = (a.Gw & 3) == 0 ? a.Gw / 4 : a.Gw;
+    const unsigned blocks = (unsigned)sm_count * 8;
+    // (how many terms there are only the device knows: at least about one per
+    // query, and one for every eight bytes of words)
+    const uint64_t terms = a.n > a.bytes_len / 8 ? a.n : a.bytes_len / 8;
+    if (terms > (uint64_t)blocks * (WORD_THREADS / 32) * WORD_ROUNDS * (pieces >= 16 ? 4 : 1)) {
+        k_probe_words_by_thread<<<blocks, WORD_THREADS, 0, s>>>(a);
+    } else {
+        uint32_t lanes = 1;
+        while (lanes < 32 && (lanes < pieces || lanes < a.eta)) lanes *= 2;
+        k_probe_words<<<blocks, WORD_THREADS, 0, s>>>(a, lanes);
+    }
     return cudaGetLastError();
 }
 

@@ -301,3 +301,35 @@ def test_few_items_in_a_large_buffer(rambo_lib, B, R):
             idx.sync()
             assert np.array_equal(rambo_lib.as_u32(got), want), (len(begins), ctas)
     assert hits > 40
+
+
+@pytest.mark.parametrize("K,B,R,eta", [
+    (60, 9, 3, 2), (60, 20, 3, 1), (60, 32, 4, 3),   # 4-, 8- and 16-byte groups: 2, 2 and 4 lanes a term
+    (60, 60, 4, 9), (60, 100, 5, 2),                 # 32 bytes and nine seeds: 16; 64 bytes: 4
+    (60, 1000, 2, 2), (40, 1000, 5, 33),             # 256 bytes: 16; two 512-byte chunks, more seeds than lanes
+])
+def test_word_queries_around_a_warp_per_term(rambo_lib, K, B, R, eta):
+    # 152 SMs x 64 warps: up to 9,728 terms have a warp each, more share it, and
+    # from 77,825 queries on (groups of 256 bytes: 311,297) a term is a thread's
+    rng = np.random.default_rng(B + eta)
+    vocab = synth.word_vocabulary(rng, 900)
+    docs = synth.word_corpus(rng, K, vocab, 60)
+    o = oracle.Rambo(K, B, R, 5003, eta, seed=5)
+    idx = rambo_lib.Index(K, B, R, 5003, eta, seed=5)
+    for d in range(K):
+        o.insert_words(d, [vocab[i] for i in docs[d]])
+    idx.insert_words(np.arange(K), [[vocab[i] for i in docs[d]] for d in range(K)])
+    # queries of a document's words, of words of none, of no word, and with empty words
+    pool = [[vocab[j] for j in rng.choice(docs[int(rng.integers(0, K))], size=int(s))] for s in rng.integers(1, 5, size=60)]
+    pool += [[], [b""], [b"", vocab[int(docs[0][0])]], [b"none of them"]]
+    want_of = [o.query_words(q) for q in pool]
+    assert np.count_nonzero(want_of) > 30
+    for terms in (1, 9727, 9728, 9729, 20_011, 800_000 if B == 1000 else 300_000):
+        pick, t = [], 0
+        while t < terms:
+            i = int(rng.integers(0, len(pool)))
+            if t + len(pool[i]) <= terms:
+                pick.append(i)
+                t += len(pool[i])
+        got = idx.query_words([pool[i] for i in pick])
+        assert np.array_equal(got, np.stack([want_of[i] for i in pick])), terms

@@ -128,3 +128,19 @@ for K, B, R, tab, n, bases in [(40_000, 250, 8, 1, 3000, 170), (40_000, 250, 8, 
     idx.close()
 """)
     assert lines == ["True", "False", "False", "False", "True", "False", "False"]
+
+
+def test_word_probe_takes_threads_for_large_batches(calls):
+    lines = calls("""
+L = rambo.load()
+z = np.zeros(10, np.uint8)
+for B, n, nbytes in [(32, 1000, 6000), (32, 77_824, 10), (32, 77_825, 10), (32, 1000, 8 * 77_825), (1000, 77_825, 10), (1000, 311_297, 10)]:
+    idx = rambo.Index(64, B, 2, 256, 2)
+    offs = np.zeros(n + 1, np.uint64)
+    out, ws = np.zeros((n, idx.W), np.uint32), aligned(L.rambo_query_words_workspace(idx._h, n))
+    log()
+    rambo._check(L.rambo_query_words_dev(idx._h, n, ptr(z), nbytes, ptr(offs), ptr(offs), ptr(out), ptr(ws), ws.size, None), "q")
+    print("k_probe_words_by_thread" in log().decode())
+    idx.close()
+""")
+    assert lines == ["False", "False", "True", "True", "False", "True"]
