@@ -333,3 +333,22 @@ def test_word_queries_around_a_warp_per_term(rambo_lib, K, B, R, eta):
                 t += len(pool[i])
         got = idx.query_words([pool[i] for i in pick])
         assert np.array_equal(got, np.stack([want_of[i] for i in pick])), terms
+
+
+def test_word_answers_that_are_held_are_not_page_locked(rambo_lib):
+    import torch
+    idx = rambo_lib.Index(300, 20, 3, 5003, 2)
+    docs = [[b"w%d" % i, b"all"] for i in range(300)]
+    idx.insert_words(np.arange(300), docs)
+    pinned = lambda a: torch.from_numpy(a.view(np.int32)).is_pinned()
+    held = [idx.query_words([[b"w%d" % i], [b"all"]]) for i in range(20)]
+    assert sum(pinned(a) for a in held) <= 1
+    part = held[0][1:]  # a view keeps the whole block
+    held = [a.copy() for a in held]
+    later = [idx.query_words([[b"w%d" % i], [b"all"]]) for i in range(20)]
+    assert not any(pinned(a) for a in later)
+    for i, (a, b) in enumerate(zip(held, later)):
+        assert np.array_equal(a, b) and i in rambo_lib.answer_docs(a[0]) and rambo_lib.answer_docs(a[1]).size == 300
+    assert rambo_lib.answer_docs(part[0]).size == 300
+    del part
+    assert pinned(idx.query_words([[b"all"]]))  # nothing is held: no copy
