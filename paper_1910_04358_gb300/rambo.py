@@ -146,6 +146,14 @@ def _stream_handle(stream):
     return stream.cuda_stream
 
 
+def _torch_stream(stream):
+    """`stream` for torch.cuda.stream(): any object with a cuda_stream handle."""
+    import torch
+    if stream is None or isinstance(stream, torch.cuda.Stream):
+        return stream
+    return torch.cuda.ExternalStream(stream.cuda_stream)
+
+
 class Workspace:
     """A 256-byte aligned device buffer owned by torch, grown on demand."""
 
@@ -426,7 +434,7 @@ class Index:
             offs = h[at:at + 8 * (len(of) + 1)].view(np.int64)
             offs[0] = 0
             np.cumsum(np.fromiter(map(len, of), dtype=np.int64, count=len(of)), out=offs[1:])
-        with torch.cuda.stream(stream):
+        with torch.cuda.stream(_torch_stream(stream)):
             buf = host.to("cuda", non_blocking=True)
         p = buf.data_ptr()
         return buf, p, p + t0, p + i0, len(text)
@@ -446,7 +454,7 @@ class Index:
         buf, text, toffs, iterms, nbytes = self._word_batch(queries, stream)
         n = len(queries)
         s = _stream_handle(stream)
-        with torch.cuda.stream(stream):
+        with torch.cuda.stream(_torch_stream(stream)):
             out = torch.empty((n, self.W), dtype=torch.int32, device="cuda")
             need = int(load().rambo_query_words_workspace(self._h, n))
             wp, wn = self._workspace(("words", s), need)

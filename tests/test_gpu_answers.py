@@ -352,3 +352,17 @@ def test_word_answers_that_are_held_are_not_page_locked(rambo_lib):
     assert rambo_lib.answer_docs(part[0]).size == 300
     del part
     assert pinned(idx.query_words([[b"all"]]))  # nothing is held: no copy
+
+
+def test_words_on_any_stream(rambo_lib):
+    # a stream is whatever has its handle, as for every other call
+    import types
+
+    import torch
+    idx = rambo_lib.Index(30, 10, 3, 5003, 2)
+    side = torch.cuda.Stream()
+    for i, stream in enumerate((None, side, torch.cuda.ExternalStream(side.cuda_stream),
+                                types.SimpleNamespace(cuda_stream=side.cuda_stream))):
+        idx.insert_words([i], [[b"word%d" % i]], stream=stream)
+        got = idx.query_words([[b"word%d" % i], []], stream=stream)
+        assert i in rambo_lib.answer_docs(got[0]) and rambo_lib.answer_docs(got[1]).size == i + 1
