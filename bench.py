@@ -34,7 +34,7 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-from paper_1910_04358_gb300.autotune import effective_path  # noqa: E402  (no torch, no library)
+from paper_1910_04358_gb300.autotune import effective_path, ran_path  # noqa: E402  (no torch, no library)
 
 METRIC = "k-mer queries/s and query bp/s on 1 GB300 (bit-exact vs oracle); serving p50/p99 ms"
 UNIT = "k-mer queries/s"
@@ -666,7 +666,7 @@ def run_sharded(args):
     dom_ms = prof["probe_seqs"]["ms"] / max(prof["probe_seqs"]["timed"], 1)
     info = idx.info
     alg_bytes = probe_algorithmic_bytes(info, n_seq_kmers, q.n, q.n_bases)
-    if effective_path(idx.get_tuning(), info) == 1:
+    if ran_path(effective_path(idx.get_tuning(), info), prof) == 1:
         alg_bytes += q.n * idx.W * 4
     peak, peak_src = measured_peak_gbs()
     achieved = alg_bytes / (dom_ms / 1e3) / 1e9
@@ -935,9 +935,7 @@ def run_ours(args):
     dom = "probe_seqs" if q.n else "probe_kmers"
     dom_ms = prof[dom]["ms"] / max(prof[dom]["timed"], 1)
     alg_bytes = probe_algorithmic_bytes(info, n_seq_kmers, q.n, q.n_bases)
-    path = effective_path(idx.get_tuning(), info)
-    if path == 1 and info["group_bytes"] <= 16:
-        path = 0  # one-lane groups take the separate launches
+    path = ran_path(effective_path(idx.get_tuning(), info), prof)
     if path == 1:  # the fused launch also writes the answer masks
         alg_bytes += q.n * idx.W * 4
     peak, peak_src = measured_peak_gbs()

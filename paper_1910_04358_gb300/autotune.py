@@ -9,8 +9,8 @@ expansion grid and byte-table policy.  It times the batch under each
 candidate with CUDA events on the launching stream and insists that every
 candidate returns exactly the same answer bits as the first one (the knobs
 change launch shapes only).  Search: for every query path that this index
-geometry actually runs (a requested path the library cannot take for these
-groups falls back to another, and is then not a separate candidate), a
+geometry and batch actually run (a requested path the library does not take
+for them falls back to another, and is then not a separate candidate), a
 coordinate descent over the other knobs, one knob at a time in the order of
 KNOBS, keeping the best value before moving on, repeated while a whole pass
 still improves (at most three passes); the best of the paths wins.
@@ -61,11 +61,13 @@ def _time(run, reps: int):
 
 
 def effective_path(tuning, info) -> int:
-    """Sequence query path the library takes for this tuning and geometry (the
-    binding always passes a workspace large enough for paths 2 and 3, and
-    batches as CSR offsets): the binned path for groups of at most 64 bytes,
-    the content-ordered path for groups of at most 64 bytes and eta <= 4, the
-    fused path for groups of at most 512 bytes, else the separate launches."""
+    """Sequence query path that this tuning and geometry ask for (the binding
+    always passes a workspace large enough for paths 2 and 3, and batches as CSR
+    offsets): the binned path for groups of at most 64 bytes, the content-ordered
+    path for groups of at most 64 bytes and eta <= 4, the fused path for groups of
+    at most 512 bytes, else the separate launches.  The library runs the fused
+    path's small batches and one-lane groups as separate launches too, by rules on
+    the batch: `ran_path` tells from the launches."""
     g = info["group_bytes"]
     if tuning["query_path"] == 2 and g <= 64:
         return 2
@@ -76,7 +78,27 @@ def effective_path(tuning, info) -> int:
     return 0
 
 
-def _descend(idx, run, outputs, ref, start, knobs, reps, info, trials, verbose, passes: int = 3):
+def ran_path(path: int, profile) -> int:
+    """`path` (of effective_path) as the library ran it, from the launch counts
+    since a profile_reset: the persistent launch expands its own answers, the
+    separate launches have an expansion.  (Groups that reach the fused path
+    answer single k-mers without one.)"""
+    return 0 if path == 1 and profile["expand"]["launches"] else path
+
+
+def _path_of(idx, run, start) -> int:
+    """The path that the batch takes under the tuning `start`."""
+    path = effective_path(start, idx.info)
+    if path != 1 or not hasattr(idx, "profile_reset"):
+        return path
+    idx.set_tuning(**start)
+    idx.profile_reset()
+    run()
+    idx.sync()
+    return ran_path(path, idx.profile_read())
+
+
+def _descend(idx, run, outputs, ref, start, path, knobs, reps, trials, verbose, passes: int = 3):
     """Coordinate descent from `start` over `knobs`, repeated while a whole
     pass still improves (at most `passes`: a knob tuned early may want
     another value once a later one has moved); returns (best, ms)."""
@@ -84,7 +106,6 @@ def _descend(idx, run, outputs, ref, start, knobs, reps, info, trials, verbose, 
     idx.set_tuning(**start)
     best_cfg, best_ms = dict(start), _time(run, reps)
     trials.append({"tuning": dict(start), "ms": best_ms})
-    path = effective_path(start, info)
     for _ in range(passes):
         before = dict(best_cfg)
         best_cfg, best_ms = _one_pass(idx, run, outputs, ref, best_cfg, best_ms, knobs, reps, path, trials,
@@ -131,7 +152,6 @@ def autotune(idx, run, outputs, reps: int = 7, knobs=KNOBS, verbose: bool = Fals
     {"best": tuning, "ms": best time, "trials": [...]}.
     """
     base = idx.get_tuning()
-    info = idx.info
     run()
     idx.sync()
     ref = [t.clone() for t in outputs()]
@@ -140,14 +160,14 @@ def autotune(idx, run, outputs, reps: int = 7, knobs=KNOBS, verbose: bool = Fals
     starts, seen = [], set()
     for qp in paths:
         start = dict(base, query_path=qp)
-        ep = effective_path(start, info)
-        if ep not in seen:
-            seen.add(ep)
-            starts.append(start)
+        path = _path_of(idx, run, start)
+        if path not in seen:
+            seen.add(path)
+            starts.append((start, path))
     trials, best = [], None
     try:
-        for start in starts:
-            cfg, ms = _descend(idx, run, outputs, ref, start, rest, reps, info, trials, verbose)
+        for start, path in starts:
+            cfg, ms = _descend(idx, run, outputs, ref, start, path, rest, reps, trials, verbose)
             if best is None or ms < best[1]:
                 best = (cfg, ms)
     except Exception:

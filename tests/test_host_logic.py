@@ -165,3 +165,33 @@ def test_a_warp_holds_a_whole_insert_record():
             assert 1 <= lanes <= 32, (R, B, g.Gw)
             by_word += bits > 0
     assert by_word > 100
+
+
+def test_autotune_and_bench_go_by_the_path_that_ran(monkeypatch):
+    # a batch of path 1 that the library runs as separate launches: no candidate
+    # of its own, and the fused knobs, which then do nothing, are left alone
+    import torch
+    from paper_1910_04358_gb300 import autotune
+
+    class Index(_FakeIndex):
+        persistent = False
+
+        def profile_reset(self, timed_stages=()):
+            pass
+
+        def profile_read(self):
+            on = self.persistent and autotune.effective_path(self.t, self.info) == 1
+            return {"probe_seqs": {"launches": 3 if on else 1}, "expand": {"launches": 0 if on else 1}}
+
+    out = torch.zeros(4, dtype=torch.int32)
+    for persistent in (False, True):
+        idx = Index(256)
+        idx.persistent = persistent
+        monkeypatch.setattr(autotune, "_time", lambda run, reps: _fused_cost(idx.t, idx.info))
+        res = autotune.autotune(idx, lambda: None, lambda: [out], reps=1)
+        tuned = {(t["tuning"]["query_path"], t["tuning"]["fused_tile_kmers"]) for t in res["trials"]}
+        assert (1 in {p for p, _ in tuned}) == persistent
+        assert (len({k for _, k in tuned}) > 1) == persistent
+    launches = lambda n: {"expand": {"launches": n}}
+    assert [autotune.ran_path(p, launches(0)) for p in range(4)] == [0, 1, 2, 3]
+    assert [autotune.ran_path(p, launches(5)) for p in range(4)] == [0, 0, 2, 3]
