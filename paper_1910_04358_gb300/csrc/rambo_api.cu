@@ -552,7 +552,12 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
         RAMBO_TRY(launch_fused(a, e, g, qs, go, h->sm_count, s));
         return RAMBO_OK;
     }
-    const uint32_t tile = probe_tile_kmers(n, packed_bytes * 4, h->sm_count);
+    // (beside k-mer chunks, whose copies out bound a host call, even tiles: blocks
+    // of small ones queue up before the chunks' blocks; 3,000 sequences of 1 kbp
+    // and 200,000 k-mers on 256-byte groups 846 against 753 us with three chunks
+    // at once, 840 against 790..810 with four)
+    const bool few = fused_ctas_cap == 0 && probe_few_items(n, packed_bytes * 4, h->sm_count);
+    const uint32_t tile = probe_tile_kmers(few, packed_bytes * 4, h->sm_count);
     {
         StageScope sc(h, RAMBO_STAGE_PREFIX, s, kmer_prefix_launches(n));
         RAMBO_TRY(launch_kmer_prefix(offsets, ends, n, g.k, packed_bytes, kcum, bsum, h->d_err, s, tile, 0, acc,
@@ -577,7 +582,7 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
     a.err = h->d_err;
     a.min_chunk = h->tune.probe_min_kmers_per_warp;
     a.max_kmers = packed_bytes * 4;
-    a.few = probe_few_items(n, packed_bytes * 4, h->sm_count);
+    a.few = few;
     {
         StageScope sc(h, RAMBO_STAGE_PROBE_SEQS, s, 1);
         RAMBO_TRY(launch_probe_seqs(a, g, tile, probe_grid(h), s));
@@ -586,9 +591,11 @@ int query_seqs_enqueue(rambo_t *h, uint64_t n, const uint8_t *packed, uint64_t p
 }
 
 // few_blocks: the answers go straight to host memory beside a sequence branch.
-// A block an SM over all chunks in flight keeps the link busy; more of them
-// clog the way of the sequences' gathers (medium batch with host buffers, 38
-// blocks a chunk: 0.80 ms, 76: 0.83, 152: 0.85, 304: 0.87..1.19).
+// A quarter of a block an SM for a chunk keeps the link busy, however many
+// chunks are in flight; more blocks clog the way of the sequences' gathers
+// (medium batch with host buffers, four chunks in flight, 38 blocks each: 0.80
+// ms, 76: 0.83, 152: 0.85, 304: 0.87..1.19; three chunks, 38 or 51 blocks: 0.80
+// and 0.81; one, 38 or 152: 1.31 and 1.33).
 int query_kmers_enqueue(rambo_t *h, uint64_t n, const uint64_t *kmers, uint32_t *out, void *ws,
                         cudaStream_t s, bool few_blocks = false) {
     const Geometry &g = h->g;

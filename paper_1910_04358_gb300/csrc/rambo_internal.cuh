@@ -199,7 +199,7 @@ struct ProbeArgs {
     uint32_t *err;
     uint32_t min_chunk;      // minimum k-mers per warp (0 = default)
     uint64_t max_kmers;      // sequence batch: about how many k-mers it has (grid sizing only)
-    uint32_t few;            // separate probe launch: probe_few_items
+    uint32_t few;            // separate probe launch: cut as a batch of few items (probe_few_items)
 };
 
 struct ExpandArgs {
@@ -311,8 +311,8 @@ cudaError_t launch_fold(const uint32_t *old_index, uint32_t old_gw, uint32_t *ne
 // 333), and a few places in a large buffer would be cut as if they were all of
 // it.  Their tiles are small, and warps take several.
 bool probe_few_items(uint64_t n, uint64_t max_kmers, int sm_count);
-// k-mers per tile of a batch of n items in a buffer of max_kmers k-mers
-uint32_t probe_tile_kmers(uint64_t n, uint64_t max_kmers, int sm_count);
+// k-mers per tile of a batch in a buffer of max_kmers k-mers
+uint32_t probe_tile_kmers(bool few, uint64_t max_kmers, int sm_count);
 // kcum: the batch's tile prefix (launch_kmer_prefix, `tile`); acc set to ones
 cudaError_t launch_probe_seqs(const ProbeArgs &a, const Geometry &g, uint32_t tile, int sm_count, cudaStream_t s);
 // (groups of 512 bytes and more; the others are probed by launch_kmer_answers)

@@ -251,8 +251,8 @@ bool probe_few_items(uint64_t n, uint64_t max_kmers, int sm_count) {
 
 // 1,024 (of 16 or more rounds of loads), fewer when that leaves warps without
 // a tile.
-uint32_t probe_tile_kmers(uint64_t n, uint64_t max_kmers, int sm_count) {
-    if (probe_few_items(n, max_kmers, sm_count)) return SEQ_TILE;
+uint32_t probe_tile_kmers(bool few, uint64_t max_kmers, int sm_count) {
+    if (few) return SEQ_TILE;
     const uint64_t t = max_kmers / ((uint64_t)sm_count * SEQ_RESIDENT) / 64 * 64;
     return (uint32_t)(t < SEQ_TILE ? SEQ_TILE : t > SEQ_TILE_MAX ? SEQ_TILE_MAX : t);
 }

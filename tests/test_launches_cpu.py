@@ -144,3 +144,16 @@ for B, n, nbytes in [(32, 1000, 6000), (32, 77_824, 10), (32, 77_825, 10), (32, 
     idx.close()
 """)
     assert lines == ["False", "False", "True", "True", "False", "True"]
+
+
+def test_sequences_beside_kmer_chunks_of_a_host_call_keep_even_tiles(calls):
+    lines = calls("""
+idx = rambo.Index(100, 100, 5, 256, 2)
+n = 3000
+packed, offs = np.zeros(n * 1000 // 4, np.uint8), np.arange(n + 1, dtype=np.uint64) * 1000
+for kmers in (np.zeros(0, np.uint64), np.zeros(100, np.uint64)):
+    log()
+    idx.query_batch(kmers, packed, offs)
+    print([l for l in log().decode().splitlines() if "k_probe_tiles" in l][0])
+""")
+    assert ["Lb1E" in line for line in lines] == [True, False]  # the instance for few items, or not
