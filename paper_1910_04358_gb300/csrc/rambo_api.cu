@@ -675,6 +675,7 @@ int insert_enqueue(rambo_t *h, uint64_t n, const uint32_t *doc_ids, const uint8_
     a.pattern = h->d_pattern;
     a.kind = !h->d_pattern ? 0 : g.Gw > 1 ? 1 : 2;
     a.lanes = a.kind == 0 ? (g.R < 32 ? g.R : 32) : g.Gw > 1 ? g.Gw / 2 : 1;
+    a.max_kmers = ends == offsets + 1 ? packed_bytes * 4 : 0;  // (ranges may overlap)
     uint32_t rshift = 0;
     uint32_t nbins =
         h->tune.insert_mode == 3 && h->d_bins && ends == offsets + 1

@@ -229,6 +229,7 @@ struct InsertArgs {
     uint32_t kind;             // RecordSetter: 0 = a lane per repetition, 1 = per 64-bit word,
                                // 2 = one 32-bit word
     uint32_t lanes;            // lanes per record, 1..32
+    uint64_t max_kmers;        // the batch has at most so many (grid sizing only); 0: not known
 };
 
 // Word documents (Section 5.4): term t is bytes [term_offs[t], term_offs[t+1])

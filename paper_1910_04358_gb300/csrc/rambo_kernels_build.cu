@@ -400,7 +400,12 @@ int blocks_per_sm(KernelT kernel, int threads) {
 template <int ETA, int KIND>
 cudaError_t launch_insert_k(const InsertArgs &a, int sm_count, cudaStream_t s) {
     static int occ = blocks_per_sm(k_insert<ETA, KIND>, INSERT_THREADS);
-k_insert<ETA, KIND><<<sm_count * occ * INSERT_WAVES, INSERT_THREADS, 0, s>>>(a);
+    uint64_t blocks = (uint64_t)sm_count * occ * INSERT_WAVES;
+    // a warp takes 64 k-mers and more: a small batch needs no more blocks than that
+    // (a document of 60 bases, 64-byte groups: 36 us with all of them, 30)
+    const uint64_t need = (a.max_kmers + INSERT_THREADS * 2 - 1) / (INSERT_THREADS * 2);
+    if (a.max_kmers && blocks > need) blocks = need;
+    k_insert<ETA, KIND><<<(unsigned)blocks, INSERT_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 

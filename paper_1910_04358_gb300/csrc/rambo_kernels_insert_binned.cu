@@ -24,7 +24,8 @@ namespace rgpu {
 namespace {
 
 constexpr int IB_THREADS = 256;
-constexpr uint32_t IB_UNIT = 2048;  // records per unit of the apply pass
+constexpr uint32_t IB_UNIT = 2048;     // records per unit of the apply pass
+constexpr uint32_t IB_UNIT_MIN = 128;  // ... of a small batch, at least
 
 __device__ __forceinline__ uint32_t record_group(unsigned long long rec) { return (uint32_t)(rec >> IB_DOC_BITS); }
 __device__ __forceinline__ uint32_t record_doc(unsigned long long rec) {
@@ -269,7 +270,11 @@ __device__ __forceinline__ void copy_once(void *smem, const void *gmem, uint64_t
 
 constexpr size_t apply_smem(size_t pattern) { return (size_t)IB_RING * IB_UNIT * 8 + pattern; }
 
-template <int KIND, bool SPAT>
+// SMALL: units of fewer records where the batch has less than one of IB_UNIT for
+// every CTA; a thousand records in a warp wait for one another's latency (10^5
+// k-mers on 64-byte groups: the whole insertion 102 us in full units, 61 so; the
+// counts made by variables cost the medium build 2%, so it has its own template).
+template <int KIND, bool SPAT, bool SMALL>
 __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, BinnedInsert b) {
     extern __shared__ uint4 ib_apply_smem[];
     unsigned long long *ring = reinterpret_cast<unsigned long long *>(ib_apply_smem);  // IB_RING x IB_UNIT
@@ -277,11 +282,24 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, B
     __shared__ uint32_t s_pre[IB_MAX_BINS + 1];  // units before bin i
     __shared__ uint32_t s_unit[IB_RING + 1];     // claimed units
     __shared__ uint32_t s_have[IB_RING];         // records of the staged units
+    // records per unit: IB_UNIT; SMALL: less when that leaves CTAs without one
+    uint32_t unit = IB_UNIT;
+    if constexpr (SMALL) {
+        __shared__ uint32_t s_total;  // records of all bins (fewer than 2^32: see the launch)
+        if (threadIdx.x == 0) s_total = 0;
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < b.nbins; i += IB_THREADS) {
+            const uint64_t n = b.count[i] < b.cap ? b.count[i] : b.cap;
+            if (n) atomicAdd(&s_total, (uint32_t)n);
+        }
+        __syncthreads();
+        while (unit > IB_UNIT_MIN && s_total < (uint64_t)gridDim.x * unit) unit /= 2;
+    }
     // units per bin, then their exclusive prefix (warp 0: lane l sums bins
     // l*PER .. l*PER + PER - 1, a warp scan, then each lane writes its run)
     for (uint32_t i = threadIdx.x; i < b.nbins; i += IB_THREADS) {
         const uint64_t n = b.count[i] < b.cap ? b.count[i] : b.cap;
-        s_pre[i] = (uint32_t)((n + IB_UNIT - 1) / IB_UNIT);
+        s_pre[i] = (uint32_t)((n + unit - 1) / unit);
     }
     if (SPAT)
         for (uint32_t i = threadIdx.x; i < a.K * a.lanes; i += IB_THREADS) s_pattern[i] = __ldg(a.pattern + i);
@@ -326,8 +344,8 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, B
                 else hi = mid;
             }
             const uint64_t n = b.count[lo] < b.cap ? b.count[lo] : b.cap;
-            const uint64_t r0 = (uint64_t)(u - s_pre[lo]) * IB_UNIT;
-            const uint32_t have = n - r0 < IB_UNIT ? (uint32_t)(n - r0) : IB_UNIT;
+            const uint64_t r0 = (uint64_t)(u - s_pre[lo]) * unit;
+            const uint32_t have = n - r0 < unit ? (uint32_t)(n - r0) : unit;
             unsigned long long *to = ring + j % IB_RING * IB_UNIT;
             const unsigned long long *from = b.buf + (uint64_t)lo * b.cap + r0;
             // pairs of records (bins hold an even number of slots)
@@ -339,8 +357,8 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, B
     for (uint32_t j = 0; j + 1 < IB_RING; ++j) fetch(j);
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t per = 32 / a.lanes, sub = lane / a.lanes, part = lane - sub * a.lanes;
-    constexpr uint32_t SHARE = IB_UNIT / (IB_THREADS / 32);  // records of a unit per warp
-    const uint32_t w0 = (threadIdx.x >> 5) * SHARE;
+    const uint32_t share = (SMALL ? unit : IB_UNIT) / (IB_THREADS / 32);  // records of a unit per warp
+    const uint32_t w0 = (threadIdx.x >> 5) * share;
     uint32_t next = 0;
     for (uint32_t j = 0;; ++j) {
         if (s_unit[j % (IB_RING + 1)] >= units) break;  // the whole CTA (claims increase)
@@ -353,7 +371,7 @@ __global__ void __launch_bounds__(IB_THREADS) k_insert_bin_apply(InsertArgs a, B
         if (threadIdx.x == 0) next = atomicAdd(claim, 1u);
         const unsigned long long *rec = ring + j % IB_RING * IB_UNIT + w0;
         const uint32_t have = s_have[j % IB_RING];
-        const uint32_t n = have > w0 ? (have - w0 < SHARE ? have - w0 : SHARE) : 0u;
+        const uint32_t n = have > w0 ? (have - w0 < share ? have - w0 : share) : 0u;
         if (sub < per) {
 #pragma unroll 4
             for (uint32_t i = sub; i < n; i += per) {
@@ -399,20 +417,31 @@ cudaError_t launch_scatter(const InsertArgs &a, const BinnedInsert &b, uint64_t 
                            cudaStream_t s) {
     const auto kernel = k_insert_bin_scatter<ETA, KIND>;
     const int occ = ib_blocks_per_sm(kernel, scatter_smem(), scatter_smem());
-    kernel<<<sm_count * occ * SCATTER_WAVES, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
+    uint64_t blocks = (uint64_t)sm_count * occ * SCATTER_WAVES;
+    const uint64_t last = a.max_kmers && a.max_kmers < f1 ? a.max_kmers : f1;
+    const uint64_t tiles = (last - f0 + IB_TILE_RECORDS / ETA - 1) / (IB_TILE_RECORDS / ETA);  // (f0 < max_kmers)
+    if (blocks > tiles) blocks = tiles;
+    kernel<<<(unsigned)blocks, IB_THREADS, scatter_smem(), s>>>(a, b, f0, f1);
     return cudaGetLastError();
 }
 
 // Patterns of up to this many bytes go to shared memory.
 constexpr uint64_t IB_PATTERN_MAX = 32 * 1024;
 
-template <int KIND, bool SPAT>
-cudaError_t launch_apply(const InsertArgs &a, const BinnedInsert &b, int sm_count, cudaStream_t s) {
-    const auto kernel = k_insert_bin_apply<KIND, SPAT>;
+template <int KIND, bool SPAT, bool SMALL>
+cudaError_t launch_apply_t(const InsertArgs &a, const BinnedInsert &b, int sm_count, cudaStream_t s) {
+    const auto kernel = k_insert_bin_apply<KIND, SPAT, SMALL>;
     const size_t smem = apply_smem(SPAT ? (size_t)a.K * a.lanes * 8 : 0);
     const int occ = ib_blocks_per_sm(kernel, smem, apply_smem(SPAT ? IB_PATTERN_MAX : 0));
     kernel<<<sm_count * occ, IB_THREADS, smem, s>>>(a, b);
     return cudaGetLastError();
+}
+
+template <int KIND, bool SPAT>
+cudaError_t launch_apply(const InsertArgs &a, const BinnedInsert &b, int sm_count, cudaStream_t s) {
+    // (five resident blocks an SM at most: 48 KB of shared memory each)
+    const bool small = a.max_kmers && a.max_kmers < (uint64_t)sm_count * 5 * IB_UNIT / a.eta;
+    return small ? launch_apply_t<KIND, SPAT, true>(a, b, sm_count, s) : launch_apply_t<KIND, SPAT, false>(a, b, sm_count, s);
 }
 
 template <int KIND>

@@ -366,3 +366,30 @@ def test_words_on_any_stream(rambo_lib):
         idx.insert_words([i], [[b"word%d" % i]], stream=stream)
         got = idx.query_words([[b"word%d" % i], []], stream=stream)
         assert i in rambo_lib.answer_docs(got[0]) and rambo_lib.answer_docs(got[1]).size == i + 1
+
+
+@pytest.mark.parametrize("K,B,R,eta", [
+    (50, 9, 3, 2),       # 4-byte groups
+    (200, 31, 4, 1),     # 16 bytes, patterns in shared memory
+    (3000, 31, 4, 2),    # ... and too many documents for it
+    (120, 100, 5, 3),    # 64 bytes, a lane per repetition
+])
+def test_binned_insertion_around_its_small_batches(rambo_lib, K, B, R, eta):
+    # batches of few k-mers are applied in smaller units, from 5 units of 2,048
+    # records an SM on in full ones; few and many documents, one of them long
+    import torch
+    edge = 152 * 5 * 2048 // eta
+    rng = np.random.default_rng(K)
+    packed = torch.from_numpy(rng.integers(0, 256, size=edge // 2 + 64, dtype=np.uint8)).cuda()
+    for bases in (31, 5000, 60_000, edge - 8, edge + 8, 2 * edge):
+        cuts = np.sort(rng.integers(0, bases + 1, size=min(K, bases // 200 + 1) - 1))
+        offs = torch.from_numpy(np.concatenate([[0], cuts, [bases]]).astype(np.int64)).cuda()
+        ids = torch.from_numpy(rng.permutation(K)[:offs.numel() - 1].astype(np.int32)).cuda()
+        got = []
+        for st in (dict(insert_mode=2), dict(insert_mode=3, bin_region_kib=64), dict(insert_mode=3, bin_region_kib=512)):
+            with rambo_lib.Index(K, B, R, 1 << 15, eta, 31, 3) as idx:
+                idx.set_tuning(**st)
+                idx.insert_batch_dev(ids, packed[:(bases + 3) // 4], offs)
+                idx.sync()
+                got.append(idx.copy_index())
+        assert got[0].any() and np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2]), bases

@@ -157,3 +157,23 @@ for kmers in (np.zeros(0, np.uint64), np.zeros(100, np.uint64)):
     print([l for l in log().decode().splitlines() if "k_probe_tiles" in l][0])
 """)
     assert ["Lb1E" in line for line in lines] == [True, False]  # the instance for few items, or not
+
+
+def test_insertion_grids_of_small_batches(calls):
+    # no more blocks than the k-mers that the buffer can hold give work to
+    lines = calls("""
+idx = rambo.Index(100, 100, 5, 256, 2)
+for mode in (2, 3):
+    idx.set_tuning(insert_mode=mode)
+    for bases in (60, 100_000, 400_000_000):
+        if bases > 1_000_000 and mode == 2:
+            continue
+        L, z, offs = rambo.load(), np.zeros(10, np.uint8), np.zeros(3, np.uint64)
+        ids, ws = np.zeros(2, np.uint32), aligned(idx.workspace_bytes("insert", 2))
+        log()
+        rambo._check(L.rambo_insert_batch_dev(idx._h, 2, ptr(ids), ptr(z), bases // 4, ptr(offs), ptr(ws), ws.size, None), "i")
+        print([l for l in log().decode().splitlines() if l.startswith("launch") and "k_insert" in l][0])
+""")
+    blocks = [int(re.search(r"grid=(\d+),1 ", line).group(1)) for line in lines]
+    assert "k_insert_bin_scatter" in lines[2]
+    assert blocks == [1, 196, 1, 49, 152 * 3 * 16]
