@@ -124,10 +124,11 @@ def test_persistent_launch_beside_kmer_chunks_of_a_host_call(rambo_lib, K, B, R,
 
 
 @pytest.mark.parametrize("use_byte_table", [0, 1])
-def test_expansion_of_groups_past_the_slot_tables(rambo_lib, use_byte_table):
+@pytest.mark.parametrize("K", [90, 1025, 2049, 4097, 8200])  # one, two, four and eight words a lane, and more
+def test_expansion_of_groups_past_the_slot_tables(rambo_lib, K, use_byte_table):
     # R * B of 16,384 and more: answers row by row, or through the byte table
-    rng, corpus, q, o, idx = _case(rambo_lib, 90, 4100, 4, 2, [0, 30, 31, 40, 90, 200] * 20, m=1 << 11, doc_len=80)
+    rng, corpus, q, o, idx = _case(rambo_lib, K, 4100, 4, 2, [0, 30, 31, 40, 90, 200] * 20, m=1 << 11, doc_len=80)
     kmers = synth.sample_kmers(rng, corpus, 200, 31, 0.7)
-    idx.set_tuning(use_byte_table=use_byte_table, byte_table_max_mb=64)
+    idx.set_tuning(use_byte_table=use_byte_table, byte_table_max_mb=4096)
     assert np.array_equal(idx.query_seqs(q.packed, q.offsets), o.query_seqs(q.packed, q.offsets))
     assert np.array_equal(idx.query_kmers(kmers), o.query_kmers(kmers))
