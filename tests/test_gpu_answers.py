@@ -27,13 +27,15 @@ GEOMETRIES = [
     (90, 16383, 1, 2),
     (90, 16384, 1, 2),
 ]
+# repetitions taken four pairs at a time until no query has the documents
+MANY_REPETITIONS = [(300, 6, 16, 2), (300, 6, 17, 1), (129, 9, 31, 2), (1000, 20, 128, 3), (70, 40, 200, 5)]
 
 
 def _dev(torch, a, dt):
     return torch.from_numpy(np.ascontiguousarray(a).view(dt)).cuda()
 
 
-@pytest.mark.parametrize("K,B,R,eta", GEOMETRIES)
+@pytest.mark.parametrize("K,B,R,eta", GEOMETRIES + MANY_REPETITIONS)
 def test_answers_match_oracle(rambo_lib, K, B, R, eta):
     import torch
     p = synth.Params(K=K, B=B, R=R, m=1 << 11, eta=eta, k=15, seed=K)
