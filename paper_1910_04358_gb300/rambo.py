@@ -223,7 +223,7 @@ class Index:
         self.W = info.mask_words
         self.device = info.device
         self._ws = {}
-        self._words_out = None  # weak reference to the page-locked answers handed out last
+        self._words_out = []  # weak references to page-locked answers handed out
 
     # ------------------------------------------------------------ lifetime
     def close(self):
@@ -463,14 +463,15 @@ class Index:
             host = torch.empty((n, self.W), dtype=torch.int32, pin_memory=True)
             host.copy_(out, non_blocking=True)
         self.sync(stream)
-        # The page-locked block itself is handed out while no earlier one is in
-        # use (every view of it keeps `res` alive), so that callers that drop their
-        # answers copy nothing; held answers are in ordinary memory (1,000 answers
-        # of 2.2 KB: 415 us dropped; held 543 us, 628 with a new page-locked block
-        # for each).
+        # The page-locked block itself is handed out while fewer than two earlier
+        # ones are in use (every view of one keeps its `res` alive), so that callers
+        # who drop their answers, the last ones with the next call's return, copy
+        # nothing; held answers are in ordinary memory (1,000 answers of 2.2 KB: 415
+        # us dropped; held 543 us, 628 with a new page-locked block for each).
         res = host.numpy()
-        if self._words_out is None or self._words_out() is None:
-            self._words_out = weakref.ref(res)
+        self._words_out = [r for r in self._words_out if r() is not None]
+        if len(self._words_out) < 2:
+            self._words_out.append(weakref.ref(res))
         else:
             res = np.empty((n, self.W), dtype=np.int32)
             torch.from_numpy(res).copy_(host)
