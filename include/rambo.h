@@ -344,9 +344,10 @@ typedef struct {
     uint32_t query_path;               /* sequence queries: 0 = prefix scan + probe +  */
                                        /* expand launches; 1 = persistent fused launch */
                                        /* with length-bucketed work queues (groups up  */
-                                       /* to 512 B; otherwise, and for small batches   */
-                                       /* and groups up to 16 B without early_exit,    */
-                                       /* path 0 is used); 2 =                         */
+                                       /* to 512 B; otherwise, and without early_exit  */
+                                       /* for small batches and groups up to 16 B,     */
+                                       /* some of wide answers excepted, path 0 is     */
+                                       /* used); 2 =                                   */
                                        /* region-binned probing (groups up to 64 B    */
                                        /* and a workspace from                         */
                                        /* rambo_query_seqs_workspace_for; otherwise    */
